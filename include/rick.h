@@ -295,7 +295,7 @@ rick_status rick_bin_layout(const rick_plan *plan, rick_bin_view *out);
  * bin offsets and the work lists -- but keeps its temporaries (the
  * per-visibility ranks and fractional offsets, the histogram, the scan
  * temporaries and the weight-sum partials) in a fixed array compiled into the
- * library (about 11.6 MB, held on every GPU that loads the library until the
+ * library (about 13.8 MB, held on every GPU that loads the library until the
  * process exits) instead of in ws_dev's scratch regions.  It calls no
  * cudaMalloc, cudaFree or allocating library routine.
  * The paper has no counterpart; this is an interface convenience.
@@ -318,9 +318,10 @@ rick_status rick_bin_values(rick_plan *plan, const void *vis_dev, const float *w
 /* Gridding (Eq. 3): planes[k][a_y + jy][a_x + jx] +=
  * vis w G(jx - h - fx) G(jy - h - fy) for every record, with the
  * checkerboard (-1)^(i+j) of the centred FFT folded in.  Every element of
- * planes_dev (complex64 [n_w][n][n]) is overwritten.  Each uv-tile is summed
- * in shared memory and written once (plain stores; tiles with more records
- * than one chunk add their chunk sums with float atomics).  The kernel
+ * planes_dev (complex64 [n_w][n][n]) is overwritten.  Records are summed
+ * in shared memory, by subtiles of 16 x 16 corners, and the sums added to the
+ * cleared planes with float atomics (compensated and deterministic plans: by
+ * uv-tiles, each written once unless it has more records than one chunk).  The kernel
  * weights G are degree-8 polynomial fits per unit segment (FP64 fit at plan
  * creation, FP32 evaluation).  rick_grid and rick_degrid use a word of the
  * workspace header as a work counter: calls that share a workspace must not

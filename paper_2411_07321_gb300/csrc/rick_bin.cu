@@ -91,8 +91,12 @@ static cudaError_t scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32
 // n_vis: records (inputs, or twice the inputs with the Hermitian mirror).
 __global__ void bin_init_kernel(WsHeader *hdr, uint64_t n_vis, uint32_t chunk_cap, int given,
                                 uint64_t wmin_key, uint64_t wmax_key, uint32_t n_key_blocks,
-                                const WsHeader *range_src, uint64_t n_src, int mirror)
+                                const WsHeader *range_src, uint64_t n_src, int mirror,
+                                uint32_t sub_cap)
 {
+    hdr->sub_cap = sub_cap;
+    hdr->n_items = 0;
+    hdr->n_groups = 0;
     hdr->n_vis = n_vis;
     hdr->n_src = n_src;
     hdr->mirror = (uint32_t)mirror;
@@ -247,6 +251,7 @@ struct KeyArgs {
     const double *chan_scale;
     int64_t n_src;            // inputs; records i >= n_src mirror input i - n_src (n_vis = 2 n_src)
     uint32_t wait_polls;      // limit of the wait for the block's bulk copies
+    SubShape sub;
     WsPtrs ws;
 };
 
@@ -367,7 +372,7 @@ __global__ void __launch_bounds__(RICK_KEY_THREADS) bin_key_kernel(KeyArgs a)
 #pragma unroll 2
     for (int it = 0; it < RICK_KEY_ITEMS; ++it) {
         int64_t i = base + (int64_t)it * RICK_KEY_THREADS;
-        uint32_t key = 0xFFFFFFFFu;
+        uint32_t key = 0xFFFFFFFFu, sid = 0xFFFFFFFFu;
         const int li = it * RICK_KEY_THREADS + threadIdx.x;  // index inside the block
         if (i < a.n_vis) {
             double u = s_uvw[3 * li], v = s_uvw[3 * li + 1], w = s_uvw[3 * li + 2];
@@ -391,6 +396,7 @@ __global__ void __launch_bounds__(RICK_KEY_THREADS) bin_key_kernel(KeyArgs a)
                     uint32_t cls = ex ? (ey ? 2u : 1u) : (ey ? 3u : 0u);
                     key = (((k * a.nt + (uint32_t)(ay >> a.log2T)) * a.nt +
                             (uint32_t)(ax >> a.log2T)) << 2) | cls;
+                    sid = rick_sub_id(a.sub, key, (uint32_t)lx, (uint32_t)ly);
                     a.ws.cell[i] = (uint32_t)ax | ((uint32_t)ay << 16);
                     a.ws.frac[i] = make_float2(fx, fy);
                     if (a.n_corr == 1) {
@@ -405,16 +411,14 @@ __global__ void __launch_bounds__(RICK_KEY_THREADS) bin_key_kernel(KeyArgs a)
             }
             a.ws.key[i] = key;
         }
-        // histogram, on this block's sub-counter of the bin: one atomic per run
-        // of equal keys in consecutive lanes (consecutive inputs -- the
-        // channels of one baseline and time -- mostly share a key).  The
-        // counter's old value ranks the run inside the (bin, sub-counter)
-        // range, so the scatter needs no atomics of its own.
-        const unsigned starts = run_starts(key, lane);
+        // histogram: one atomic per run of equal sub-bins in consecutive lanes
+        // (consecutive inputs -- the channels of one baseline and time -- mostly
+        // share one).  The counter's old value ranks the run inside the sub-bin,
+        // so the scatter needs no atomics of its own.
+        const unsigned starts = run_starts(sid, lane);
         uint32_t base = 0;
-        if (key != 0xFFFFFFFFu && ((starts >> lane) & 1u))
-            base = atomicAdd(&a.ws.hist[key * RICK_BIN_SUBS + (blockIdx.x & (RICK_BIN_SUBS - 1))],
-                             (uint32_t)(run_end(starts, lane) - lane));
+        if (sid != 0xFFFFFFFFu && ((starts >> lane) & 1u))
+            base = atomicAdd(&a.ws.hist[sid], (uint32_t)(run_end(starts, lane) - lane));
         const int first = run_begin(starts, lane);
         base = __shfl_sync(FULL, base, first);
         if (i < a.n_vis) a.ws.rank[i] = base + (uint32_t)(lane - first);
@@ -491,9 +495,11 @@ __global__ void __launch_bounds__(1024) bin_finalize_kernel(WsHeader *hdr, const
 template <bool CORR, bool MIRROR>
 __global__ void __launch_bounds__(256) bin_scatter_kernel(int64_t n_vis, const float2 *vis,
                                                           const float *weight, WsPtrs ws,
-                                                          int n_corr, int64_t n_src)
+                                                          int n_corr, int64_t n_src,
+                                                          SubShape sub)
 {
     constexpr int U = RICK_SCATTER_U;
+    const uint32_t tmask = (1u << sub.log2T) - 1;
     const int64_t step = (int64_t)gridDim.x * blockDim.x * U;
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x * U; i0 < n_vis; i0 += step) {
         int64_t idx[U];
@@ -534,10 +540,8 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(int64_t n_vis, const f
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (key[u] != 0xFFFFFFFFu) {
-                // the sub-counter of the key pass's block that held this input
-                const uint32_t sub = (uint32_t)((idx[u] / (RICK_KEY_THREADS * RICK_KEY_ITEMS)) &
-                                                (RICK_BIN_SUBS - 1));
-                const uint32_t pos = ws.suboff[key[u] * RICK_BIN_SUBS + sub] + rk[u];
+                const uint32_t sid = rick_sub_id(sub, key[u], cl[u] & tmask, cl[u] >> 16 & tmask);
+                const uint32_t pos = ws.suboff[sid] + rk[u];
                 ws.perm[pos] = (uint32_t)idx[u];
                 ws.rec[pos] = make_float4(v[u].x * wt[u], v[u].y * wt[u], fr[u].x, fr[u].y);
                 ws.rcell[pos] = cl[u];
@@ -546,13 +550,14 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(int64_t n_vis, const f
     }
 }
 
-// Bin offsets from the sub-counter offsets: bin b starts where its first
-// sub-range starts.
-__global__ void bin_offsets_kernel(const uint32_t *suboff, uint32_t *offsets, int64_t nbins)
+// Bin offsets from the sub-bin offsets: bin b starts where its first sub-bin
+// starts.
+__global__ void bin_offsets_kernel(const uint32_t *suboff, uint32_t *offsets, int64_t nbins,
+                                   SubShape sub)
 {
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= nbins;
          b += (int64_t)gridDim.x * blockDim.x)
-        offsets[b] = suboff[b * RICK_BIN_SUBS];
+        offsets[b] = suboff[(b >> 2) * sub.per + rick_sub_first(sub, (uint32_t)b & 3u)];
 }
 
 // Re-pack record values for new visibilities through an existing permutation,
@@ -848,6 +853,70 @@ __global__ void tile_count_kernel(const uint32_t *off, uint32_t *gcnt, uint32_t 
     dcnt[t] = (own + cap - 1) / cap;
 }
 
+// Append entries (s0 + lane of the owner, first[owner] + step i) for the cnt of
+// every lane to a list, i < cnt: one atomic per warp, all lanes writing.
+__device__ __forceinline__ void append_items(uint32_t cnt, uint32_t from, uint32_t step, uint32_t s0,
+                                             uint32_t *counter, uint2 *list)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += v;
+    }
+    const uint32_t tot = __shfl_sync(FULL, inc, 31), first = inc - cnt;
+    if (!tot) return;
+    uint32_t at = 0;
+    if (lane == 31) at = atomicAdd(counter, tot);
+    at = __shfl_sync(FULL, at, 31);
+    for (uint32_t i0 = 0; i0 < tot; i0 += 32) {
+        // entry i belongs to the last lane whose entries start at or before it
+        const uint32_t i = i0 + lane;
+        int own = 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            own += __shfl_sync(FULL, first, own + o) <= i ? o : 0;
+        const uint32_t k = i - __shfl_sync(FULL, first, own);
+        const uint32_t c = __shfl_sync(FULL, from, own) + step * k;
+        if (i < tot) list[at + i] = make_uint2(s0 + own, c);
+    }
+}
+
+// The plain gridding kernel's work items, in no particular order: a thread per
+// subtile counts its records (its class-0 sub-bin and, in the last column and
+// row of subtiles, those of the other classes).
+__global__ void __launch_bounds__(256) sub_items_kernel(const uint32_t *suboff, uint32_t nsubtiles,
+                                                        SubShape sub, WsHeader *hdr, uint2 *items,
+                                                        uint2 *groups)
+{
+    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t cnt = 0;
+    if (s < nsubtiles) {
+        uint32_t n = 0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int64_t id = rick_subtile_range(sub, s, g);
+            if (id >= 0) n += suboff[id + 1] - suboff[id];
+        }
+        cnt = rick_sub_chunks(n, hdr->sub_cap);
+    }
+    const uint32_t s0 = s - (threadIdx.x & 31), ng = cnt / RICK_SUB_GROUP;
+    append_items(ng, 0, RICK_SUB_GROUP, s0, &hdr->n_groups, groups);
+    append_items(cnt - ng * RICK_SUB_GROUP, ng * RICK_SUB_GROUP, 1, s0, &hdr->n_items, items);
+}
+
+static rick_status build_items(rick_plan *plan, const WsPtrs &w, const WsLayout &L, cudaStream_t st)
+{
+    if (!rick_grid_plain(&plan->p)) return RICK_OK;
+    const SubShape sub = rick_sub_shape(plan->p.tile);
+    const uint32_t ns = (uint32_t)(L.ntiles << (2 * sub.lq));
+    sub_items_kernel<<<(ns + 255) / 256, 256, 0, st>>>(w.suboff, ns, sub, w.hdr, w.items,
+                                                     w.groups);
+    RICK_LAUNCH_CHECK(plan);
+    return RICK_OK;
+}
+
 // ------------------------------------------------------------------------
 
 // Rows of n_chan channels that fit a plan's capacity.
@@ -881,6 +950,7 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     const int64_t nkb = (n_vis + RICK_KEY_THREADS * RICK_KEY_ITEMS - 1) /
                         (RICK_KEY_THREADS * RICK_KEY_ITEMS);
     WsPtrs w = rick_ws_ptrs(ws_dev, L);
+    const SubShape sub = rick_sub_shape(p.tile);
     cudaStream_t st = (cudaStream_t)stream;
     const bool det = (p.options & RICK_OPT_DETERMINISTIC) != 0;
     uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms);
@@ -897,7 +967,8 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     bin_init_kernel<<<1, 1, 0, st>>>(w.hdr, (uint64_t)n_vis, cap, given,
                                      isnan(p.w_min) ? 0 : rick_dkey(p.w_min),
                                      isnan(p.w_min) ? 0 : rick_dkey(p.w_max), (uint32_t)nkb,
-                                     range_src, (uint64_t)n_src, mirror);
+                                     range_src, (uint64_t)n_src, mirror,
+                                     rick_sub_cap(n_vis, plan->num_sms));
     RICK_LAUNCH_CHECK(plan);
     if (!given && n_vis > 0) {
         int blocks = plan->num_sms * 4;
@@ -909,7 +980,7 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     }
     bin_setup_kernel<<<1, 1, 0, st>>>(w.hdr, w.bkey, w.wplane, p.n_w);
     RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, cudaMemsetAsync(w.hist, 0, 4 * (size_t)(RICK_BIN_SUBS * L.nbins + 1), st));
+    RICK_CUDA_TRY(plan, cudaMemsetAsync(w.hist, 0, 4 * (size_t)(L.nsubs + 1), st));
 
     if (n_vis > 0) {
         KeyArgs ka;
@@ -932,6 +1003,7 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
         ka.chan_scale = chan_scale;
         ka.n_src = mirror ? n_src : n_vis;
         ka.wait_polls = plan->wait_polls;
+        ka.sub = sub;
         ka.bulk = n_chan == 0 && n_corr == 1 && ((uintptr_t)uvw & 15) == 0 &&
                   ((uintptr_t)weight & 15) == 0;
         const size_t smem = key_pass_smem(p.n_w);
@@ -943,10 +1015,10 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     }
     bin_finalize_kernel<<<1, 1024, 0, st>>>(w.hdr, w.wpart, (int)nkb, weight == NULL ? n_corr : 0);
     RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, RICK_BIN_SUBS * L.nbins + 1, w.scan, st,
+    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, L.nsubs + 1, w.scan, st,
                                  &plan->launches));
     bin_offsets_kernel<<<(unsigned)((L.nbins + 256) / 256), 256, 0, st>>>(w.suboff, w.offsets,
-                                                                          L.nbins);
+                                                                          L.nbins, sub);
     RICK_LAUNCH_CHECK(plan);
     if (det) {
         rick_status ds = det_sort_records(plan, w, L, n_vis, vis, weight, n_corr,
@@ -957,13 +1029,13 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
         if (blocks > (int64_t)plan->num_sms * 64) blocks = (int64_t)plan->num_sms * 64;
         if (n_corr > 1)
             bin_scatter_kernel<true, false><<<(unsigned)blocks, 256, 0, st>>>(
-                n_vis, (const float2 *)vis, weight, w, n_corr, n_vis);
+                n_vis, (const float2 *)vis, weight, w, n_corr, n_vis, sub);
         else if (mirror)
             bin_scatter_kernel<false, true><<<(unsigned)blocks, 256, 0, st>>>(
-                n_vis, (const float2 *)vis, weight, w, 1, n_src);
+                n_vis, (const float2 *)vis, weight, w, 1, n_src, sub);
         else
             bin_scatter_kernel<false, false><<<(unsigned)blocks, 256, 0, st>>>(
-                n_vis, (const float2 *)vis, weight, w, 1, n_vis);
+                n_vis, (const float2 *)vis, weight, w, 1, n_vis, sub);
         RICK_LAUNCH_CHECK(plan);
     }
     uint32_t nt = (uint32_t)L.ntiles;
@@ -972,6 +1044,10 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     RICK_LAUNCH_CHECK(plan);
     RICK_CUDA_TRY(plan, scan_u32(w.gbase, w.gbase, L.ntiles + 1, w.scan, st, &plan->launches));
     RICK_CUDA_TRY(plan, scan_u32(w.dbase, w.dbase, L.ntiles + 1, w.scan, st, &plan->launches));
+    {
+        const rick_status is = build_items(plan, w, L, st);
+        if (is != RICK_OK) return is;
+    }
     if (det) {  // slots of the tiles with several grid work items
         det_mc_flags_kernel<<<(nt + 256) / 256, 256, 0, st>>>(w.gbase, w.mcslot, nt);
         RICK_LAUNCH_CHECK(plan);
@@ -1054,12 +1130,12 @@ extern "C" rick_status rick_bin_values(rick_plan *plan, const void *vis, const f
 // ------------------------------------------------------------------------
 // rick_bin_noalloc: the binning above for callers that must not allocate
 // device memory.  Its temporaries -- the per-visibility ranks and fractional
-// offsets, the histogram / cursor array, the scan temporaries and the
-// weight-sum partials -- live in this file-scope array instead of the
+// offsets, the histogram, the scan temporaries and the weight-sum
+// partials -- live in this file-scope array instead of the
 // caller's workspace.  The per-visibility keys and corner cells stay in the
 // caller's workspace, where rick_bin writes them: degridding and the density
 // weights read them after the binning.  The array is part of the library
-// image: every GPU that loads librick.so holds it (about 11.6 MB) until the
+// image: every GPU that loads librick.so holds it (about 13.8 MB) until the
 // process exits.
 
 #define NOALLOC_MAX_VIS (1 << 18)
@@ -1067,8 +1143,8 @@ extern "C" rick_status rick_bin_values(rick_plan *plan, const void *vis, const f
 #define NOALLOC_FRAC (0)
 #define NOALLOC_RANK (NOALLOC_FRAC + 8 * NOALLOC_MAX_VIS)
 #define NOALLOC_HIST (NOALLOC_RANK + 4 * NOALLOC_MAX_VIS)
-#define NOALLOC_SUBOFF (NOALLOC_HIST + 4 * (RICK_BIN_SUBS * NOALLOC_MAX_BINS + 256))
-#define NOALLOC_SCAN (NOALLOC_SUBOFF + 4 * (RICK_BIN_SUBS * NOALLOC_MAX_BINS + 256))
+#define NOALLOC_MAX_SUBS (81 * (NOALLOC_MAX_BINS / 4))  // tile 128: 81 sub-bins per tile of 4 bins
+#define NOALLOC_SCAN (NOALLOC_HIST + 4 * (NOALLOC_MAX_SUBS + 256))
 #define NOALLOC_WPART (NOALLOC_SCAN + 4 * 4096)
 #define NOALLOC_BYTES (NOALLOC_WPART + 8 * (NOALLOC_MAX_VIS / (RICK_KEY_THREADS * RICK_KEY_ITEMS) + 256))
 
@@ -1123,10 +1199,10 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     // outputs (records, offsets, work lists, and the keys and corner cells that
     // later calls read) in the caller's workspace, temporaries in the fixed array
     WsPtrs w = rick_ws_ptrs(ws_dev, L);
+    const SubShape sub = rick_sub_shape(p.tile);
     w.rank = (uint32_t *)(scratch + NOALLOC_RANK);
     w.frac = (float2 *)(scratch + NOALLOC_FRAC);
     w.hist = (uint32_t *)(scratch + NOALLOC_HIST);
-    w.suboff = (uint32_t *)(scratch + NOALLOC_SUBOFF);
     w.scan = (uint32_t *)(scratch + NOALLOC_SCAN);
     w.wpart = (double *)(scratch + NOALLOC_WPART);
     cudaStream_t st = (cudaStream_t)stream;
@@ -1136,7 +1212,8 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     // the same stages as rick_bin, in the same order
     bin_init_kernel<<<1, 1, 0, st>>>(w.hdr, (uint64_t)n_vis, cap, given,
                                      given ? rick_dkey(p.w_min) : 0, given ? rick_dkey(p.w_max) : 0,
-                                     (uint32_t)nkb, NULL, (uint64_t)n_vis, 0);
+                                     (uint32_t)nkb, NULL, (uint64_t)n_vis, 0,
+                                     rick_sub_cap(n_vis, plan->num_sms));
     RICK_LAUNCH_CHECK(plan);
     if (!given && n_vis > 0) {
         wrange_kernel<false><<<plan->num_sms * 4, 256, 0, st>>>(uvw, n_vis, w.hdr, 0, NULL);
@@ -1145,7 +1222,7 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     bin_setup_kernel<<<1, 1, 0, st>>>(w.hdr, w.bkey, w.wplane, p.n_w);
     RICK_LAUNCH_CHECK(plan);
     // the array keeps the last call's contents: the histogram must start at zero
-    RICK_CUDA_TRY(plan, cudaMemsetAsync(w.hist, 0, 4 * (size_t)(RICK_BIN_SUBS * L.nbins + 1), st));
+    RICK_CUDA_TRY(plan, cudaMemsetAsync(w.hist, 0, 4 * (size_t)(L.nsubs + 1), st));
     if (n_vis > 0) {
         KeyArgs ka;
         ka.n_vis = n_vis;
@@ -1167,6 +1244,7 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
         ka.chan_scale = NULL;
         ka.n_src = n_vis;
         ka.wait_polls = plan->wait_polls;
+        ka.sub = sub;
         ka.bulk = ((uintptr_t)uvw & 15) == 0 && ((uintptr_t)weight & 15) == 0;
         const size_t smem = key_pass_smem(p.n_w);
         RICK_CUDA_TRY(plan, cudaFuncSetAttribute(bin_key_kernel,
@@ -1177,16 +1255,16 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     }
     bin_finalize_kernel<<<1, 1024, 0, st>>>(w.hdr, w.wpart, (int)nkb, weight == NULL);
     RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, RICK_BIN_SUBS * L.nbins + 1, w.scan, st,
+    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, L.nsubs + 1, w.scan, st,
                                  &plan->launches));
     bin_offsets_kernel<<<(unsigned)((L.nbins + 256) / 256), 256, 0, st>>>(w.suboff, w.offsets,
-                                                                          L.nbins);
+                                                                          L.nbins, sub);
     RICK_LAUNCH_CHECK(plan);
     if (n_vis > 0) {
         int64_t blocks = (n_vis + 256 * RICK_SCATTER_U - 1) / (256 * RICK_SCATTER_U);
         if (blocks > (int64_t)plan->num_sms * 64) blocks = (int64_t)plan->num_sms * 64;
         bin_scatter_kernel<false, false><<<(unsigned)blocks, 256, 0, st>>>(
-            n_vis, (const float2 *)vis, weight, w, 1, n_vis);
+            n_vis, (const float2 *)vis, weight, w, 1, n_vis, sub);
         RICK_LAUNCH_CHECK(plan);
     }
     uint32_t nt = (uint32_t)L.ntiles;
@@ -1195,6 +1273,10 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     RICK_LAUNCH_CHECK(plan);
     RICK_CUDA_TRY(plan, scan_u32(w.gbase, w.gbase, L.ntiles + 1, w.scan, st, &plan->launches));
     RICK_CUDA_TRY(plan, scan_u32(w.dbase, w.dbase, L.ntiles + 1, w.scan, st, &plan->launches));
+    {
+        const rick_status is = build_items(plan, w, L, st);
+        if (is != RICK_OK) return is;
+    }
     if (stats_dev)
         RICK_CUDA_TRY(plan, cudaMemcpyAsync(stats_dev, &w.hdr->stats, sizeof(rick_bin_stats),
                                             cudaMemcpyDeviceToDevice, st));

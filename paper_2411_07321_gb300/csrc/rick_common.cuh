@@ -122,24 +122,102 @@ struct WsHeader {
     // deterministic mode: tile sums in fixed point, value = integer * fx_inv
     float fx_scale, fx_inv;             // 2^k and 2^-k
     uint32_t mc_count;                  // tiles gridded by several work items
+    // plain gridding: records per chunk; work items and the work counters,
+    // of a warp and of a CTA
+    uint32_t sub_cap, n_items, item_next, n_groups, group_next;
 };
 
 struct WsLayout {
     size_t header, key, rank, cell, frac, perm, rec, rcell, hist, suboff, offsets, gbase, dbase, scan,
-        wpart, bkey, wplane, dkey, didx, dkey2, dcnt, vpart, mcslot, mcacc, total;
-    int64_t n_vis, nbins, ntiles, nscan, nkeyblocks, ndetblocks;
+        wpart, bkey, wplane, dkey, didx, dkey2, dcnt, vpart, mcslot, mcacc, items, groups, total;
+    int64_t n_vis, nbins, nsubs, nitems, ngroups, ntiles, nscan, nkeyblocks, ndetblocks;
 };
 
 // Key pass blocks: 1024 visibilities, staged in 28 KB of shared memory, so that
 // six blocks fit an SM (the pass is bound by integer issue and needs the warps).
 #define RICK_KEY_THREADS 256
 #define RICK_KEY_ITEMS 4
-// Each bin's histogram counter is split into RICK_BIN_SUBS sub-counters, chosen
-// by the input's block of RICK_KEY_THREADS * RICK_KEY_ITEMS visibilities: the
-// densest bins (the array core) then take their atomics on several addresses
-// instead of one.  The value a counter held before an input's atomic is the
-// input's rank within its (bin, sub-counter) range.
-#define RICK_BIN_SUBS 8
+// Sub-bins.  The records of a bin are grouped by the subtile -- S x S cells of
+// the tile, S = min(16, T) -- that holds their footprint corner: the unit of
+// work of the plain gridding kernel.  A tile has q x q subtiles (q = T / S) and
+// (q + 1)^2 sub-bins, in record order: those of edge class 0 (one per subtile,
+// row-major), of class 1 (its corners lie in the last column of subtiles, as a
+// support is at most 16: one per row of subtiles), of class 2 (the last subtile)
+// and of class 3 (one per column).  The histogram counts sub-bins; the value a
+// counter held before an input's atomic is the input's rank in its sub-bin.
+// Several counters per sub-bin, to spread the atomics of the densest ones, gain
+// nothing (LOFAR-like 5e7 visibilities: key pass 593 us with one counter per
+// bin, 596 with eight, 597 with 32).
+#define RICK_SUB_LOG 4
+
+struct SubShape {
+    int log2T, ls, lq, per;  // tile side, subtile side, subtiles per side (logs); sub-bins per tile
+};
+
+RICK_HD SubShape rick_sub_shape(int tile)
+{
+    SubShape s;
+    s.log2T = 0;
+    while ((1 << s.log2T) < tile) ++s.log2T;
+    s.ls = s.log2T < RICK_SUB_LOG ? s.log2T : RICK_SUB_LOG;
+    s.lq = s.log2T - s.ls;
+    s.per = ((1 << s.lq) + 1) * ((1 << s.lq) + 1);
+    return s;
+}
+
+// First sub-bin of an edge class.
+RICK_HD uint32_t rick_sub_first(const SubShape &s, uint32_t cls)
+{
+    const uint32_t q = 1u << s.lq;
+    return cls == 0 ? 0u : q * q + (cls == 1 ? 0u : cls == 2 ? q : q + 1);
+}
+
+// Sub-bin of a record: its bin key and the corner inside its tile.  Every plan
+// whose planes fit a GPU has fewer than 2^32 sub-bins.
+RICK_HD uint32_t rick_sub_id(const SubShape &s, uint32_t key, uint32_t lx, uint32_t ly)
+{
+    const uint32_t q = 1u << s.lq, r = ly >> s.ls, c = lx >> s.ls, cls = key & 3u;
+    const uint32_t sub = cls == 0 ? r * q + c : q * q + (cls == 1 ? r : cls == 2 ? q : q + 1 + c);
+    return (key >> 2) * (uint32_t)s.per + sub;
+}
+
+// Sub-bin g (0: its class-0 one; 1, 2, 3: those of the edge classes, in the last
+// column and row of subtiles) of subtile id = tile q^2 + row q + column, or -1.
+RICK_HD int64_t rick_subtile_range(const SubShape &s, uint32_t id, int g)
+{
+    const uint32_t q = 1u << s.lq, tile = id >> (2 * s.lq), r = id >> s.lq & (q - 1), c = id & (q - 1);
+    const int64_t base = (int64_t)tile * s.per;
+    if (g == 0) return base + r * q + c;
+    if (g == 1) return c == q - 1 ? base + q * q + r : -1;
+    if (g == 2) return c == q - 1 && r == q - 1 ? base + q * q + q : -1;
+    return r == q - 1 ? base + q * q + q + 1 + c : -1;
+}
+
+// Work of the plain gridding kernel: a subtile's records in chunks of at most
+// sub_cap, cut evenly.  Eight chunks of a subtile make a CTA's item -- a warp
+// each, summed across the warps before they go to the planes -- and what is left
+// a warp's items.  (Every chunk by itself puts hundreds of partial sums, one
+// after the other, onto the cells of the array core: the image of 2e8
+// visibilities on 8192^2 was then 4.5 times further from its 64-bit value.)
+// About four chunks per resident warp.  At most 2048 records, where the partial
+// sums are few enough (2e8 visibilities, 512 / 1024 / 2048 records: error of the
+// image 2.5e-5 / 1.3e-5 / 1.1e-5; 1.3e-5 with CTA tiles of 20559 records).  At
+// least 128, where items begin to cost more in list and reductions than they
+// balance (1e6 visibilities, 128 / 64: 50 / 55 us), or 64 for the small sets, where
+// an item's steps are the call's latency (1e4 visibilities, 64 / 128 / 512: 21 /
+// 31 / 96 us).
+#define RICK_SUB_GROUP 8
+#define RICK_SUB_CAP_MIN 64
+#define RICK_SUB_CAP_MAX 2048
+RICK_HD uint32_t rick_sub_chunks(uint32_t n, uint32_t cap) { return (n + cap - 1) / cap; }
+static inline uint32_t rick_sub_cap(int64_t n_vis, int num_sms)
+{
+    int64_t least = n_vis / ((int64_t)num_sms * 32);
+    least = least < RICK_SUB_CAP_MIN ? RICK_SUB_CAP_MIN : least > 128 ? 128 : least;
+    int64_t c = n_vis / ((int64_t)num_sms * 128);
+    c = c < least ? least : c > RICK_SUB_CAP_MAX ? RICK_SUB_CAP_MAX : c;
+    return (uint32_t)((c + 31) & ~(int64_t)31);
+}
 // Polls of a bounded device-side wait before it gives up (and the drain wait
 // of a block that gave up: its copies must land before its shared memory goes).
 #define RICK_WAIT_POLLS RICK_WAIT_POLLS_DEFAULT
@@ -195,7 +273,15 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
     L.nbins = 4 * L.ntiles;
     L.nkeyblocks = (n_vis + RICK_KEY_THREADS * RICK_KEY_ITEMS - 1) / (RICK_KEY_THREADS * RICK_KEY_ITEMS);
     L.ndetblocks = det ? (n_vis + RICK_DET_BLOCK - 1) / RICK_DET_BLOCK : 0;
-    L.nscan = rick_scan_tmp(RICK_BIN_SUBS * L.nbins + 1);
+    const SubShape sub = rick_sub_shape(p->tile);
+    L.nsubs = L.ntiles * sub.per;
+    // work items: at most one per subtile that holds records, and one more per
+    // RICK_SUB_CAP_MIN records
+    L.nitems = L.ntiles << (2 * sub.lq);
+    if (L.nitems > n_vis) L.nitems = n_vis;
+    L.nitems += n_vis / RICK_SUB_CAP_MIN + 1;
+    L.ngroups = n_vis / (RICK_SUB_GROUP - 1) / RICK_SUB_CAP_MIN + 1;
+    L.nscan = rick_scan_tmp(L.nsubs + 1);
     if (det) {
         const int64_t d = rick_scan_tmp((1 << RICK_DET_DIGIT) * L.ndetblocks + 1);
         if (d > L.nscan) L.nscan = d;
@@ -211,8 +297,8 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
     // one record of padding: the gridding loop reads one record ahead
     L.rec = o;    o += rick_align256(16 * (size_t)(nv + 1));
     L.rcell = o;  o += rick_align256(4 * (size_t)(nv + 1));
-    L.hist = o;   o += rick_align256(4 * (size_t)(RICK_BIN_SUBS * L.nbins + 1));
-    L.suboff = o; o += rick_align256(4 * (size_t)(RICK_BIN_SUBS * L.nbins + 1));
+    L.hist = o;   o += rick_align256(4 * (size_t)(L.nsubs + 1));
+    L.suboff = o; o += rick_align256(4 * (size_t)(L.nsubs + 1));
     L.offsets = o; o += rick_align256(4 * (size_t)(L.nbins + 1));
     L.gbase = o;  o += rick_align256(4 * (size_t)(L.ntiles + 1));
     L.dbase = o;  o += rick_align256(4 * (size_t)(L.ntiles + 1));
@@ -231,6 +317,8 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
     L.vpart = o;  o += rick_align256(det ? 8 * (size_t)(L.ndetblocks + 1) : 0);
     L.mcslot = o; o += rick_align256(det ? 4 * (size_t)(L.ntiles + 1) : 0);
     L.mcacc = o;  o += rick_align256(16 * (size_t)rick_det_slots(p, n_vis) * p->tile * p->tile);
+    L.items = o;  o += rick_align256(8 * (size_t)L.nitems);
+    L.groups = o; o += rick_align256(8 * (size_t)L.ngroups);
     L.total = o;
     return L;
 }
@@ -247,6 +335,7 @@ struct WsPtrs {
     uint32_t *dkey, *didx, *dkey2, *dcnt, *mcslot;  // deterministic mode
     double *vpart;
     unsigned long long *mcacc;
+    uint2 *items, *groups;  // plain gridding: (subtile, first chunk) of each work item
 };
 
 static inline WsPtrs rick_ws_ptrs(void *ws, const WsLayout &L)
@@ -277,7 +366,16 @@ static inline WsPtrs rick_ws_ptrs(void *ws, const WsLayout &L)
     w.vpart = (double *)(b + L.vpart);
     w.mcslot = (uint32_t *)(b + L.mcslot);
     w.mcacc = (unsigned long long *)(b + L.mcacc);
+    w.items = (uint2 *)(b + L.items);
+    w.groups = (uint2 *)(b + L.groups);
     return w;
+}
+
+// Plans gridded by the plain kernel, in subtiles (else by tiles: compensated
+// and deterministic sums).
+static inline bool rick_grid_plain(const rick_params *p)
+{
+    return p->precision == RICK_PREC_FP32 && !(p->options & RICK_OPT_DETERMINISTIC);
 }
 
 // Records per work item of the tile kernels for a binning of n_vis

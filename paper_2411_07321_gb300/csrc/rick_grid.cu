@@ -1,8 +1,15 @@
 // rick_grid.cu -- convolutional gridding (Eq. 3 of De Rubeis et al.) and its
 // adjoint, degridding.
 //
-// Gridding: one CTA per work item = (uv-tile of one w-plane, chunk of at most
-// chunk_cap records).  The CTA owns the T x T output cells of its tile: it sums
+// Plain gridding: one warp per work item = (subtile of one w-plane, chunk of at
+// most sub_cap records).  The warp sums the footprints of its records -- every
+// corner in the 16 x 16 cells of the subtile -- into (16 + W - 1)^2 cells of its
+// own in shared memory, with plain loads and stores, and adds the cells it
+// reached to the planes (16-byte reductions in L2) onto tiles cleared before.
+//
+// Compensated and deterministic gridding: one CTA per work item = (uv-tile of
+// one w-plane, chunk of at most chunk_cap records).  The CTA owns the T x T
+// output cells of its tile: it sums
 // into a shared-memory accumulator the records binned at the tile (footprint
 // corner inside it) and the records of the west / north / north-west tiles
 // whose footprints reach into it (their edge classes), each clipped to the
@@ -25,11 +32,14 @@ struct GridArgs {
     int accumulate;  // add into the planes instead of overwriting them
     const uint8_t *touched;  // per tile: add into it (tiles an earlier chunk gridded), or NULL
     uint32_t nzero;  // tile-clearing items (RICK_ZERO_GROUP tiles each); 0 when accumulating
+    SubShape sub;            // plain sums: subtiles, their record offsets, the work items
+    const uint32_t *suboff;
+    const uint2 *items, *groups;
     const uint32_t *mcslot;     // deterministic mode: slot of each multi-item tile
     unsigned long long *mcacc;  // deterministic mode: the slots' int64 (re, im) sums
 };
 
-// Accumulation modes of the grid kernel: FP32 shared-memory sums, FP32 rounds
+// Accumulation modes: FP32 sums (one warp per subtile), FP32 rounds
 // folded by compensated summation, or 64-bit fixed point (deterministic: the
 // sums do not depend on the order of the atomics).
 #define GM_PLAIN 0
@@ -101,6 +111,15 @@ struct StreamShape {
     static constexpr int LIVE = NG * G;  // lanes of a warp that carry a stream
 };
 
+// The cells a subtile's footprints reach, and the stride of their rows in shared
+// memory: odd, so that the lanes of a group, one row each, access 8-byte cells in
+// distinct bank pairs.
+template <int W>
+struct SubCells {
+    static constexpr int ROWS = (1 << RICK_SUB_LOG) + W - 1, STRIDE = ROWS | 1;
+    static constexpr int CELLS = ROWS * STRIDE;
+};
+
 // Warps of a gridding CTA (256 threads).
 #define RICK_GRID_WARPS 8
 
@@ -121,6 +140,19 @@ __device__ __forceinline__ void group_flush(float *acc_re, float *acc_im, int fb
             atomicAdd(&acc_im[fb + jx], ai[jx]);
         }
     }
+}
+
+// The lane's row sums into its warp's cells, fb the index of the row's first one.
+// No other warp writes them, and the groups of the warp take turns.
+template <int W>
+__device__ __forceinline__ void warp_flush(float2 *cells, int fb, const float *ar, const float *ai)
+{
+    float2 *p = cells + fb;
+    float2 o[W];
+#pragma unroll
+    for (int jx = 0; jx < W; ++jx) o[jx] = p[jx];
+#pragma unroll
+    for (int jx = 0; jx < W; ++jx) p[jx] = make_float2(o[jx].x + ar[jx], o[jx].y + ai[jx]);
 }
 
 // The same into the 64-bit fixed-point tile: each row sum scaled by 2^k and
@@ -161,12 +193,12 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // Record ring of a warp: where a warp carries at most three record streams
-// (W >= 9, three CTAs per SM), the streams' next records are staged in shared
-// memory by the whole warp, RICK_GRID_RB records per stream per chunk, two
-// chunks in flight, so that the record loop reads them from shared memory
-// instead of waiting on global loads one record ahead (large workload, W = 9:
-// grid 9.92 -> 9.06 ms).  With four streams (W = 7, four CTAs per SM) the
-// extra warps already hide the loads and the ring measured 2 % slower.
+// (W >= 9), the streams' next records are staged in shared memory by the whole
+// warp, RICK_GRID_RB records per stream per chunk, two chunks in flight, so that
+// the record loop reads them from shared memory instead of waiting on global
+// loads one record ahead.  With four streams (W = 7) the loads that the ring
+// would save are shared by more records a step, and it measured slower (5e7
+// visibilities: 1.16 -> 1.24 ms; plain loads two records ahead: 1.34).
 #define RICK_GRID_RB 16
 
 template <int W>
@@ -352,7 +384,7 @@ __device__ __forceinline__ void grid_stream(const TileArgs &ta, uint32_t r0, uin
 }
 
 template <int W, int MODE>
-__device__ __forceinline__ void grid_item(const GridArgs &a, uint32_t b, uint32_t t, float *sm,
+__device__ __forceinline__ void tile_item(const GridArgs &a, uint32_t b, uint32_t t, float *sm,
                                           const float2 *coef2)
 {
     constexpr bool COMP = MODE == GM_COMP, DET = MODE == GM_DET;
@@ -411,7 +443,7 @@ __device__ __forceinline__ void grid_item(const GridArgs &a, uint32_t b, uint32_
     }
     __syncthreads();
 
-    // plain: one round over the chunk; compensated: rounds of 4096 records,
+    // deterministic: one round over the chunk; compensated: rounds of 4096 records,
     // each folded into the (sum, compensation) pair of every cell.  The
     // round's piece of each of the four ranges is split evenly into one
     // contiguous run per record stream, so the streams of a warp always walk
@@ -436,8 +468,7 @@ __device__ __forceinline__ void grid_item(const GridArgs &a, uint32_t b, uint32_
                 const uint32_t v0 = min(a0 + stream * per, a1), v1 = min(v0 + per, a1);
                 const uint32_t nv = streaming ? v1 - v0 : 0u;
                 grid_stream<W, DET>(ta, s_rs[g] + ((nv ? v0 : a0) - base), nv, per, x0, y0,
-                                    acc_re, acc_im,
-                                        T, TP, coef2, acc64, fx);
+                                     acc_re, acc_im, T, TP, coef2, acc64, fx);
             }
             base += lg;
         }
@@ -511,25 +542,33 @@ __device__ __forceinline__ void zero_group(const GridArgs &a, uint32_t z)
     }
 }
 
+// This lane's kernel segment (= its footprint row within its group).
+template <int W>
+__device__ __forceinline__ void load_coef(const KernelPoly &kp, float2 *coef2)
+{
+    const int seg = min((int)((threadIdx.x & 31) % StreamShape<W>::G), W - 1);
+#pragma unroll
+    for (int k = 0; k < RICK_POLY_N; ++k) {
+        coef2[k] = make_float2(kp.c[seg][k], kp.c[seg][k]);
+        // opaque from here on: the compiler would rather read them again in every
+        // step than keep them, and a lane-indexed constant load is a replay per row
+        asm volatile("" : "+f"(coef2[k].x), "+f"(coef2[k].y));
+    }
+}
+
 // Persistent: one wave of CTAs takes work items (tile, chunk) from a counter
 // in the workspace header (reset by zero_tiles_kernel, launched just before),
 // and with each a clearing item for a group of tiles without records, so that
 // the HBM-bound clearing of the empty tiles runs under the issue-bound
-// gridding of the others.  Four CTAs per SM for W <= 8 (64 registers a
-// thread): the record loop is latency-bound, and the extra warps hide more of
-// it than the few spilled registers cost.
+// gridding of the others.
 template <int W, int MODE>
-__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, (W <= 8 && MODE == GM_PLAIN) ? 4 : 3)
-    grid_kernel(GridArgs a)
+__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, 3) grid_kernel(GridArgs a)
 {
     extern __shared__ float sm[];
     __shared__ uint32_t s_b, s_tile, s_z;
     const uint32_t total = a.t.base[a.t.ntiles];
-    // this lane's kernel segment (= its footprint row within its group)
-    const int seg = min((int)((threadIdx.x & 31) % StreamShape<W>::G), W - 1);
     float2 coef2[RICK_POLY_N];
-#pragma unroll
-    for (int k = 0; k < RICK_POLY_N; ++k) coef2[k] = make_float2(a.t.kp.c[seg][k], a.t.kp.c[seg][k]);
+    load_coef<W>(a.t.kp, coef2);
     for (;;) {
         if (threadIdx.x == 0) {
             const uint32_t b = atomicAdd(&a.t.hdr->grid_next, 1u);
@@ -542,10 +581,319 @@ __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, (W <= 8 && MODE == GM_PL
         __syncthreads();  // everyone has the item before thread 0 takes the next
         if (b >= total && z >= a.nzero) break;
         if (b < total) {
-            grid_item<W, MODE>(a, b, t, sm, coef2);
+            tile_item<W, MODE>(a, b, t, sm, coef2);
             __syncthreads();  // the accumulator is reused by the next item
         }
         if (z < a.nzero) zero_group(a, z);
+    }
+}
+
+// Plane and first cell of a subtile.
+struct SubOrigin {
+    int k, x0, y0;
+};
+__device__ __forceinline__ SubOrigin sub_origin(const GridArgs &a, uint32_t id)
+{
+    const SubShape &sub = a.sub;
+    const uint32_t q = 1u << sub.lq, tile = id >> (2 * sub.lq), nt = a.t.nt, row = tile / nt;
+    return {(int)(row / nt), (int)(((tile - row * nt) << sub.log2T) + ((id & (q - 1)) << sub.ls)),
+            (int)((row % nt << sub.log2T) + ((id >> sub.lq & (q - 1)) << sub.ls))};
+}
+
+// n records, r0 ... r0 + n - 1, in ntrip >= n steps (the same for every lane of the
+// warp) into the warp's cells; fbase: index of this lane's footprint row for a
+// corner at (0, 0).  As grid_stream, but for the flush.
+template <int W>
+__device__ __forceinline__ void warp_stream(const TileArgs &ta, uint32_t r0, uint32_t n,
+                                            uint32_t ntrip, int fbase, const float2 *coef2,
+                                            float2 *cells)
+{
+    constexpr int G = StreamShape<W>::G, NGR = StreamShape<W>::NG, ST = SubCells<W>::STRIDE;
+    using Ring = RecRing<W>;
+    constexpr int RB = RICK_GRID_RB, NH = (Ring::SLOTS + 31) / 32;
+    __shared__ __align__(16) float4 s_rrec[Ring::ON ? RICK_GRID_WARPS * 2 * Ring::SLOTS : 1];
+    __shared__ uint32_t s_rcel[Ring::ON ? RICK_GRID_WARPS * 2 * Ring::SLOTS : 1];
+    const int lane = threadIdx.x & 31;
+    const int grp = lane / G, j = lane - grp * G, rg = grp < NGR ? grp : NGR - 1;
+    const int lead = grp * G;
+    const bool live = lane < StreamShape<W>::LIVE && j < W && n > 0;
+    const uint32_t last = r0 + (n > 0 ? n - 1 : 0);  // absolute, as is r
+    float ar[W], ai[W];
+#pragma unroll
+    for (int jx = 0; jx < W; ++jx) ar[jx] = ai[jx] = 0.0f;
+    float4 *wrec = s_rrec + (Ring::ON ? (threadIdx.x >> 5) * 2 * Ring::SLOTS : 0);
+    uint32_t *wcel = s_rcel + (Ring::ON ? (threadIdx.x >> 5) * 2 * Ring::SLOTS : 0);
+    uint32_t cr0[NH], clast[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+        const int g = min((lane + 32 * h) / RB, NGR - 1);
+        cr0[h] = Ring::ON ? __shfl_sync(0xffffffffu, r0, g * G) : 0u;
+        clast[h] = Ring::ON ? __shfl_sync(0xffffffffu, last - r0, g * G) : 0u;
+    }
+    // ring slot of the stream's record i (idle lanes read any stream)
+    auto ring_at = [&](uint32_t i) {
+        return (int)((i / RB) & 1u) * Ring::SLOTS + rg * RB + (int)(i % RB);
+    };
+    uint32_t r = r0, cur;
+    float4 q;
+    int ri = 0;
+    if constexpr (Ring::ON) {
+        ring_issue<W>(ta, wrec, wcel, 0, cr0, clast);
+        ring_issue<W>(ta, wrec, wcel, 1, cr0, clast);
+        cp_async_wait1();
+        __syncwarp();
+        ri = ring_at(0);
+        q = wrec[ri];
+        cur = wcel[ri];
+    } else {
+        q = ta.rec[r];
+        cur = ta.rcell[r];
+    }
+    uint32_t cell = cur;
+    for (uint32_t i = 0; i < ntrip; ++i) {
+        // the next record; past the stream's end the last one again
+        float4 nq;
+        uint32_t ncell;
+        const bool in = i < n;
+        if constexpr (Ring::ON) {
+            const uint32_t i1 = i + 1;
+            if (i1 % RB == 0) {
+                if (i1 < ntrip) {
+                    // entering chunk c = i1 / RB: the warp is done with chunk c - 1
+                    // (record i was read last iteration), so its buffer takes chunk
+                    // c + 1; chunk c has landed once only that copy is pending
+                    __syncwarp();
+                    ring_issue<W>(ta, wrec, wcel, i1 / RB + 1, cr0, clast);
+                    cp_async_wait1();
+                    __syncwarp();
+                }
+                ri = ring_at(i1);
+            } else {
+                ++ri;
+            }
+            nq = wrec[ri];
+            ncell = wcel[ri];
+        } else {
+            r = min(r + 1, last);
+            nq = ta.rec[r];
+            ncell = ta.rcell[r];
+        }
+        // the groups that change corner, one after the other: footprints of two
+        // groups may overlap
+        const bool turn = cell != cur;
+        if (__any_sync(0xffffffffu, turn)) {
+            unsigned m = __ballot_sync(0xffffffffu, turn && live && j == 0);
+            while (m) {
+                if (live && grp * G == __ffs(m) - 1)
+                    warp_flush<W>(cells, (int)((cur >> 16) * ST + (cur & 0xFFFFu)) + fbase, ar, ai);
+                __syncwarp();
+                m &= m - 1;
+            }
+            if (turn) {
+#pragma unroll
+                for (int jx = 0; jx < W; ++jx) ar[jx] = ai[jx] = 0.0f;
+                cur = cell;
+            }
+        }
+        float gx = 1.0f, gy = 1.0f;
+        if (W > 1) {
+            const float2 s2 = make_float2(2.0f * (q.z - ta.kp.fc), 2.0f * (q.w - ta.kp.fc));
+            float2 g2 = coef2[RICK_POLY_DEG];
+#pragma unroll
+            for (int k = RICK_POLY_DEG - 1; k >= 0; --k) g2 = __ffma2_rn(g2, s2, coef2[k]);
+            gx = g2.x;
+            gy = g2.y;
+        }
+        const float gz = in ? gy : 0.0f;
+        const float2 vv = __fmul2_rn(make_float2(q.x, q.y), make_float2(gz, gz));
+        const float2 vr2 = make_float2(vv.x, vv.x), vi2 = make_float2(vv.y, vv.y);
+        float wv[W];
+#pragma unroll
+        for (int jx = 0; jx < W; ++jx) {
+            // power-of-two groups: the lane inside the group is an immediate
+            // (width form); groups of W lanes: the absolute lane
+            wv[jx] = W == 1 ? gx
+                   : (G & (G - 1)) == 0 ? __shfl_sync(0xffffffffu, gx, jx, G)
+                                        : __shfl_sync(0xffffffffu, gx, grp * G + jx);
+        }
+#pragma unroll
+        for (int jx = 0; jx + 1 < W; jx += 2) {
+            const float2 w2 = make_float2(wv[jx], wv[jx + 1]);
+            const float2 a2 = __ffma2_rn(vr2, w2, make_float2(ar[jx], ar[jx + 1]));
+            const float2 b2 = __ffma2_rn(vi2, w2, make_float2(ai[jx], ai[jx + 1]));
+            ar[jx] = a2.x; ar[jx + 1] = a2.y;
+            ai[jx] = b2.x; ai[jx + 1] = b2.y;
+        }
+        if (W & 1) {
+            ar[W - 1] = __fmaf_rn(vv.x, wv[W - 1], ar[W - 1]);
+            ai[W - 1] = __fmaf_rn(vv.y, wv[W - 1], ai[W - 1]);
+        }
+        q = nq;
+        cell = ncell;
+    }
+#pragma unroll 1
+    for (int h = 0; h < NGR; ++h) {
+        if (live && grp == h)
+            warp_flush<W>(cells, (int)((cur >> 16) * ST + (cur & 0xFFFFu)) + fbase, ar, ai);
+        __syncwarp();
+    }
+    if constexpr (Ring::ON) {
+        // the copies still in flight land before the ring is used again
+        cp_async_wait0();
+        __syncwarp();
+    }
+}
+
+// Chunk `chunk` of a subtile's records into the warp's cells.
+template <int W>
+__device__ __forceinline__ void grid_chunk(const GridArgs &a, uint32_t id, uint32_t chunk,
+                                           float2 *cells, const float2 *coef2)
+{
+    constexpr int NG = StreamShape<W>::NG;
+    const SubShape &sub = a.sub;
+    const int lane = threadIdx.x & 31;
+    // the subtile's up to four record ranges, lane g holding range g
+    uint32_t rs = 0, rl = 0;
+    if (lane < 4) {
+        const int64_t rid = rick_subtile_range(sub, id, lane);
+        if (rid >= 0) {
+            rs = a.suboff[rid];
+            rl = a.suboff[rid + 1] - rs;
+        }
+    }
+    uint32_t n = rl + __shfl_xor_sync(0xffffffffu, rl, 1);
+    n += __shfl_xor_sync(0xffffffffu, n, 2);
+    n = __shfl_sync(0xffffffffu, n, 0);
+    const uint32_t nch = rick_sub_chunks(n, a.t.hdr->sub_cap), len = (n + nch - 1) / nch;
+    const uint32_t vbeg = chunk * len, vend = min(vbeg + len, n);
+    const SubOrigin so = sub_origin(a, id);
+    const int fbase = (lane % StreamShape<W>::G - so.y0) * SubCells<W>::STRIDE - so.x0;
+    const bool streaming = lane < StreamShape<W>::LIVE;
+    const uint32_t stream = streaming ? lane / StreamShape<W>::G : 0;
+    uint32_t base = 0;
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+        const uint32_t s = __shfl_sync(0xffffffffu, rs, g), l = __shfl_sync(0xffffffffu, rl, g);
+        const uint32_t a0 = max(vbeg, base), a1 = min(vend, base + l);
+        if (a0 < a1) {
+            // split evenly into one run per stream
+            const uint32_t per = (a1 - a0 + NG - 1) / NG;
+            const uint32_t v0 = min(a0 + stream * per, a1), v1 = min(v0 + per, a1);
+            const uint32_t nv = streaming ? v1 - v0 : 0u;
+            warp_stream<W>(a.t, s + ((nv ? v0 : a0) - base), nv, per, fbase, coef2, cells);
+        }
+        base += l;
+    }
+}
+
+// The sums of nc sets of a subtile's cells (strides of SubCells::CELLS) added to
+// the planes and the cells zeroed, by threads t of nt: two cells of a row at a
+// time, the checkerboard (-1)^(i+j) folded in (x0, y0 and the column are even);
+// cells that no footprint reached are zero, those off the grid among them.
+template <int W>
+__device__ __forceinline__ void cells_out(const GridArgs &a, uint32_t id, float2 *cells, int nc,
+                                          int t, int nt)
+{
+    constexpr int ROWS = SubCells<W>::ROWS, ST = SubCells<W>::STRIDE, HP = (ROWS + 1) / 2;
+    const SubOrigin so = sub_origin(a, id);
+    const int n = a.t.n;
+    float2 *plane = a.planes + ((size_t)so.k * n + so.y0) * n + so.x0;
+    for (int i = t; i < ROWS * HP; i += nt) {
+        const int row = i / HP, col = 2 * (i - row * HP);
+        const bool two = ROWS % 2 == 0 || col + 1 < ROWS;
+        float2 u = make_float2(0.0f, 0.0f), v = u;
+#pragma unroll 2
+        for (int c = 0; c < nc; ++c) {
+            float2 *p = cells + c * SubCells<W>::CELLS + row * ST + col;
+            u = __fadd2_rn(u, p[0]);
+            p[0] = make_float2(0.0f, 0.0f);
+            if (two) {
+                v = __fadd2_rn(v, p[1]);
+                p[1] = make_float2(0.0f, 0.0f);
+            }
+        }
+        if (u.x != 0.0f || u.y != 0.0f || v.x != 0.0f || v.y != 0.0f) {
+            if (row & 1) {
+                u.x = -u.x;
+                u.y = -u.y;
+            } else {
+                v.x = -v.x;
+                v.y = -v.y;
+            }
+            atomicAdd((float4 *)(plane + (size_t)row * n + col), make_float4(u.x, u.y, v.x, v.y));
+        }
+    }
+}
+
+// A work item: of the CTA (a chunk per warp, one sum; all threads call it) or, with
+// single, of the warp.  cells: the CTA's.
+template <int W>
+__device__ __forceinline__ void grid_item(const GridArgs &a, bool single, uint2 item, float2 *cells,
+                                          const float2 *coef2)
+{
+    // (the subtile waits in shared memory: the record loop needs the registers)
+    __shared__ volatile uint32_t s_id[RICK_GRID_WARPS];
+    const int wid = threadIdx.x >> 5;
+    float2 *own = cells + wid * SubCells<W>::CELLS;
+    s_id[wid] = item.x;
+    grid_chunk<W>(a, item.x, item.y + (single ? 0 : wid), own, coef2);
+    if (single)
+        __syncwarp();
+    else
+        __syncthreads();
+    cells_out<W>(a, s_id[wid], single ? own : cells, single ? 1 : RICK_GRID_WARPS,
+                 single ? threadIdx.x & 31 : threadIdx.x, single ? 32 : 32 * RICK_GRID_WARPS);
+    __syncwarp();
+}
+
+// Take the next item of a counter: for the whole CTA, or for each warp.
+__device__ __forceinline__ uint32_t next_cta(uint32_t *counter)
+{
+    __shared__ uint32_t s_next;
+    __syncthreads();  // the cells are zero again, the last index has been read
+    if (threadIdx.x == 0) s_next = atomicAdd(counter, 1u);
+    __syncthreads();
+    return s_next;
+}
+__device__ __forceinline__ uint32_t next_warp(uint32_t *counter)
+{
+    uint32_t b = 0;
+    if ((threadIdx.x & 31) == 0) b = atomicAdd(counter, 1u);
+    return __shfl_sync(0xffffffffu, b, 0);
+}
+
+// Plain sums: the CTAs take the groups of chunks from a counter in the workspace
+// header (reset by zero_tiles_kernel, launched just before), then each warp takes
+// single chunks from another until none is left.
+//
+// Bound by instruction issue (62 % of cycles; long_scoreboard, the record loads,
+// is the first stall).  A warp owns its cells, so a corner change costs W loads
+// and stores of 8 bytes a lane, and only the groups meet at barriers; summing a
+// 64 x 64 tile per CTA took 2 W compare-and-swap loops a lane there (shared memory
+// has no FP32 add) and visited the records near a tile's edge once per tile they
+// reach.  16 x 16 corners a subtile leave 32 warps an SM.  On a GB300, against the
+// CTA tiles: 5e7 visibilities of 16 channels, W = 7: 1.92 -> 1.24 ms; 2e8 of 64,
+// W = 9: 9.21 -> 6.81; 1e7 of 4: 0.68 -> 0.35; 4e6 of one: 0.61 -> 0.33; 1e6 of 4:
+// 106 -> 52 us; 1e4: 58 -> 20 us.  Four CTAs an SM up to W = 10 (W = 9 at three:
+// 2 % slower).
+template <int W>
+__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
+    grid_warps_kernel(const __grid_constant__ GridArgs a)
+{
+    extern __shared__ float2 s_cells[];
+    float2 coef2[RICK_POLY_N];
+    load_coef<W>(a.t.kp, coef2);
+    for (int i = threadIdx.x; i < RICK_GRID_WARPS * SubCells<W>::CELLS; i += 32 * RICK_GRID_WARPS)
+        s_cells[i] = make_float2(0.0f, 0.0f);
+    WsHeader *hdr = a.t.hdr;
+#pragma unroll 1
+    for (int single = 0; single < 2; ++single) {
+        const uint32_t total = single ? hdr->n_items : hdr->n_groups;
+        for (;;) {
+            const uint32_t b = single ? next_warp(&hdr->item_next) : next_cta(&hdr->group_next);
+            if (b >= total) break;
+            grid_item<W>(a, single, single ? a.items[b] : a.groups[b], s_cells, coef2);
+        }
     }
 }
 
@@ -561,10 +909,23 @@ struct GridBatchArgs {
 };
 static_assert(sizeof(GridBatchArgs) <= 32764, "kernel parameters are limited to 32764 bytes");
 
-// Zero the tiles whose chunks add into them with atomics (more than one work
-// item) before the grid kernel runs, and reset the grid kernel's counters.
-// Grid-stride, one warp per tile, 16-byte stores.  Tiles without records are
-// cleared by the grid kernel itself; when gridding adds into existing planes
+// Tile t of the planes zeroed by the whole block, 16 bytes a store.
+__device__ __forceinline__ void clear_tile(float2 *planes, uint32_t t, int nt, int log2T, int n)
+{
+    const uint32_t tx = t % nt, ty = t / nt % nt, k = t / nt / nt;
+    float4 *tile = (float4 *)(planes + ((size_t)k * n + (ty << log2T)) * n + (tx << log2T));
+    const int lh = log2T - 1;  // float4 = two cells
+    for (int i = threadIdx.x; i < 1 << (log2T + lh); i += blockDim.x)
+        tile[(size_t)(i >> lh) * (n / 2) + (i & ((1 << lh) - 1))] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+#define RICK_ZERO_LOOK 8
+
+// Zero the tiles of at least `least` work items, into which the grid kernel adds,
+// before it runs, and reset its counters: least = 2 for the compensated kernel
+// (a tile's only item stores it, and the kernel itself clears the tiles without
+// records), 1 for the plain one, or 0 where every tile has to be written.
+// When gridding adds into existing planes
 // nothing is cleared, and neither are the tiles flagged in touched (a chunk of a
 // streamed set adds into the tiles earlier chunks gridded).
 // Deterministic mode (mcacc != NULL): the int64 slots of those tiles are
@@ -575,16 +936,18 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
                                                          WsHeader *hdr, int accumulate,
                                                          const uint32_t *mcslot,
                                                          unsigned long long *mcacc,
-                                                         const uint8_t *touched)
+                                                         const uint8_t *touched, uint32_t least)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hdr->grid_next = 0;
         hdr->zero_next = 0;
+        hdr->item_next = 0;
+        hdr->group_next = 0;
     }
     int lane = threadIdx.x & 31;
     uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int T = 1 << log2T, half = T >> 1;  // float4 = two cells
+    const int T = 1 << log2T;
     if (mcacc) {
         for (uint32_t t = warp; t < ntiles; t += nwarps) {
             if (base[t + 1] - base[t] <= 1) continue;
@@ -594,89 +957,77 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
         return;
     }
     if (accumulate) return;
-    for (uint32_t t = warp; t < ntiles; t += nwarps) {
-        if (base[t + 1] - base[t] <= 1 || (touched && touched[t])) continue;
-        uint32_t tx = t % nt, ty = (t / nt) % nt, k = t / (nt * nt);
-        float4 *plane = (float4 *)(planes + (size_t)k * n * n);
-        for (int i = lane; i < T * half; i += 32) {
-            int row = i / half, col2 = i - row * half;
-            plane[((size_t)((ty << log2T) + row) * n + (tx << log2T)) / 2 + col2] =
-                make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+    // a block looks at RICK_ZERO_LOOK tiles at a time, and its warps share the rows
+    // of each one to clear: the tiles with records lie side by side
+    for (uint32_t t0 = blockIdx.x * RICK_ZERO_LOOK; t0 < ntiles; t0 += gridDim.x * RICK_ZERO_LOOK) {
+        const uint32_t tl = t0 + lane;
+        unsigned m = __ballot_sync(0xffffffffu, lane < RICK_ZERO_LOOK && tl < ntiles &&
+                                                    base[tl + 1] - base[tl] >= least &&
+                                                    !(touched && touched[tl]));
+        for (; m; m &= m - 1) clear_tile(planes, t0 + __ffs(m) - 1, nt, log2T, n);
     }
 }
 
-// The batch's multi-item tiles zeroed (one row of CTAs per job, blockIdx.y) and
+// The batch's tiles with records zeroed (one row of CTAs per job, blockIdx.y) and
 // its item counter reset.
 __global__ void __launch_bounds__(256)
     zero_tiles_batch_kernel(const __grid_constant__ GridBatchArgs ba)
 {
     const GridArgs &a = ba.job[blockIdx.y];
     const TileArgs &ta = a.t;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) ta.hdr->grid_next = 0;
-    const int lane = threadIdx.x & 31, log2T = a.log2T, T = 1 << log2T, half = T >> 1;
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int nt = ta.nt, n = ta.n;
-    for (uint32_t t = warp; t < ta.ntiles; t += nwarps) {
-        if (ta.base[t + 1] - ta.base[t] <= 1) continue;
-        const uint32_t tx = t % nt, ty = (t / nt) % nt, k = t / (nt * nt);
-        float4 *plane = (float4 *)(a.planes + (size_t)k * n * n);
-        for (int i = lane; i < T * half; i += 32) {
-            const int row = i / half, col2 = i - row * half;
-            plane[((size_t)((ty << log2T) + row) * n + (tx << log2T)) / 2 + col2] =
-                make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        ta.hdr->item_next = 0;
+        ta.hdr->group_next = 0;
+    }
+    const int lane = threadIdx.x & 31;
+    for (uint32_t t0 = blockIdx.x * RICK_ZERO_LOOK; t0 < ta.ntiles;
+         t0 += gridDim.x * RICK_ZERO_LOOK) {
+        const uint32_t tl = t0 + lane;
+        unsigned m = __ballot_sync(0xffffffffu, lane < RICK_ZERO_LOOK && tl < ta.ntiles &&
+                                                    ta.base[tl + 1] != ta.base[tl]);
+        for (; m; m &= m - 1) clear_tile(a.planes, t0 + __ffs(m) - 1, ta.nt, a.log2T, ta.n);
     }
 }
 
-// Persistent over the batch's work items: item b of the list belongs to the
-// job j with cum[j] <= b < cum[j + 1] (cum: running totals of the jobs' items),
-// and is that job's item b - cum[j].  A CTA reloads its lanes' kernel
-// coefficients when the job changes.
+// As grid_warps_kernel over the batch's work: entry b of the jobs' lists belongs to
+// the job j with cum[j] <= b < cum[j + 1] (cum: running totals of the jobs'
+// entries), and is that job's entry b - cum[j].  The lanes' kernel coefficients
+// are loaded again when the job changes.
 template <int W>
-__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 8 ? 4 : 3)
+__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_batch_kernel(const __grid_constant__ GridBatchArgs ba)
 {
-    extern __shared__ float sm[];
-    __shared__ uint32_t s_cum[RICK_GRID_BATCH_MAX + 1];
-    __shared__ uint32_t s_b, s_tile, s_job;
-    if (threadIdx.x == 0) {
+    extern __shared__ float2 s_cells[];
+    __shared__ uint32_t s_cum[2][RICK_GRID_BATCH_MAX + 1];
+    if (threadIdx.x < 2) {
         uint32_t c = 0;
-        s_cum[0] = 0;
+        s_cum[threadIdx.x][0] = 0;
         for (int j = 0; j < ba.n_jobs; ++j) {
-            c += ba.job[j].t.base[ba.job[j].t.ntiles];
-            s_cum[j + 1] = c;
+            const WsHeader *h = ba.job[j].t.hdr;
+            c += threadIdx.x ? h->n_items : h->n_groups;
+            s_cum[threadIdx.x][j + 1] = c;
         }
     }
+    for (int i = threadIdx.x; i < RICK_GRID_WARPS * SubCells<W>::CELLS; i += 32 * RICK_GRID_WARPS)
+        s_cells[i] = make_float2(0.0f, 0.0f);
     __syncthreads();
-    const uint32_t total = s_cum[ba.n_jobs];
-    const int seg = min((int)((threadIdx.x & 31) % StreamShape<W>::G), W - 1);
     float2 coef2[RICK_POLY_N];
     int cur = -1;
-    for (;;) {
-        if (threadIdx.x == 0) {
-            const uint32_t b = atomicAdd(&ba.job[0].t.hdr->grid_next, 1u);
+#pragma unroll 1
+    for (int single = 0; single < 2; ++single) {
+        WsHeader *h0 = ba.job[0].t.hdr;
+        const uint32_t *cum = s_cum[single], total = cum[ba.n_jobs];
+        for (;;) {
+            const uint32_t b = single ? next_warp(&h0->item_next) : next_cta(&h0->group_next);
+            if (b >= total) break;
             int j = 0;
-            while (j + 1 < ba.n_jobs && s_cum[j + 1] <= b) ++j;
-            s_b = b;
-            s_job = (uint32_t)j;
-            s_tile = b < total ? find_tile(ba.job[j].t.base, ba.job[j].t.ntiles, b - s_cum[j]) : 0u;
-        }
-        __syncthreads();
-        const uint32_t b = s_b, t = s_tile;
-        const int j = (int)s_job;
-        __syncthreads();  // everyone has the item before thread 0 takes the next
-        if (b >= total) break;
-        const GridArgs &a = ba.job[j];
-        if (j != cur) {
-#pragma unroll
-            for (int k = 0; k < RICK_POLY_N; ++k)
-                coef2[k] = make_float2(a.t.kp.c[seg][k], a.t.kp.c[seg][k]);
+            while (j + 1 < ba.n_jobs && cum[j + 1] <= b) ++j;
+            const GridArgs &a = ba.job[j];
+            if (j != cur) load_coef<W>(a.t.kp, coef2);
             cur = j;
+            grid_item<W>(a, single, single ? a.items[b - cum[j]] : a.groups[b - cum[j]], s_cells,
+                         coef2);
         }
-        grid_item<W, GM_PLAIN>(a, b - s_cum[j], t, sm, coef2);
-        __syncthreads();  // the accumulator is reused by the next item
     }
 }
 
@@ -842,6 +1193,14 @@ static TileArgs make_tile_args(const rick_plan *plan, const WsPtrs &w, const uin
     return t;
 }
 
+static void set_sub_args(GridArgs &a, const rick_params &p, const WsPtrs &w)
+{
+    a.sub = rick_sub_shape(p.tile);
+    a.suboff = w.suboff;
+    a.items = w.items;
+    a.groups = w.groups;
+}
+
 static int ilog2(int x)
 {
     int l = 0;
@@ -863,8 +1222,8 @@ static unsigned persistent_blocks(K kernel, size_t smem, int num_sms)
 template <int W, int MODE>
 static cudaError_t launch_grid_t(const GridArgs &a, int num_sms, cudaStream_t st)
 {
-    // float words: two T (T + 1) arrays; compensated six; 64-bit sums four
-    const int words = MODE == GM_COMP ? 6 : MODE == GM_DET ? 4 : 2;
+    // float words: six T (T + 1) arrays, or four of 64-bit sums
+    const int words = MODE == GM_COMP ? 6 : 4;
     size_t smem = words * (size_t)a.t.T * (a.t.T + 1) * sizeof(float);
     cudaFuncSetAttribute(grid_kernel<W, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
@@ -874,11 +1233,23 @@ static cudaError_t launch_grid_t(const GridArgs &a, int num_sms, cudaStream_t st
 }
 
 template <int W>
+static size_t warps_smem()
+{
+    return RICK_GRID_WARPS * sizeof(float2) * SubCells<W>::CELLS;
+}
+
+template <int W>
 static cudaError_t launch_grid(const GridArgs &a, int mode, int num_sms, cudaStream_t st)
 {
-    return mode == GM_COMP ? launch_grid_t<W, GM_COMP>(a, num_sms, st)
-         : mode == GM_DET  ? launch_grid_t<W, GM_DET>(a, num_sms, st)
-                           : launch_grid_t<W, GM_PLAIN>(a, num_sms, st);
+    if (mode == GM_COMP) return launch_grid_t<W, GM_COMP>(a, num_sms, st);
+    if (mode == GM_DET) return launch_grid_t<W, GM_DET>(a, num_sms, st);
+    const size_t smem = warps_smem<W>();
+    cudaError_t e = cudaFuncSetAttribute(grid_warps_kernel<W>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    grid_warps_kernel<W><<<persistent_blocks(grid_warps_kernel<W>, smem, num_sms),
+                           32 * RICK_GRID_WARPS, smem, st>>>(a);
+    return cudaGetLastError();
 }
 
 template <int W>
@@ -935,9 +1306,11 @@ rick_status rick_grid_impl(rick_plan *plan, void *ws_dev, void *planes_dev, int 
     if (det && mode == RICK_GRID_CHUNK_TILES) return RICK_EINVAL;  // its slots add per tile
     a.mcslot = det ? w.mcslot : NULL;
     a.mcacc = det ? w.mcacc : NULL;
+    set_sub_args(a, p, w);
+    const uint32_t least = !rick_grid_plain(&p) ? 2u : mode == RICK_GRID_OVERWRITE ? 0u : 1u;
     zero_tiles_kernel<<<(accumulate && !det) ? 1 : plan->num_sms * 8, 256, 0, st>>>(
         w.gbase, a.t.ntiles, a.t.nt, a.log2T, p.n, a.planes, w.hdr, accumulate, a.mcslot,
-        a.mcacc, a.touched);
+        a.mcacc, a.touched, least);
     RICK_LAUNCH_CHECK(plan);
     const int gmode = det ? GM_DET : p.precision == RICK_PREC_FP32_COMPENSATED ? GM_COMP : GM_PLAIN;
 #define CALL_GRID(WW) err = launch_grid<WW>(a, gmode, plan->num_sms, st)
@@ -973,7 +1346,7 @@ extern "C" rick_status rick_grid_accumulate(rick_plan *plan, void *ws_dev, void 
 template <int W>
 static cudaError_t launch_grid_batch(const GridBatchArgs &ba, int num_sms, cudaStream_t st)
 {
-    const size_t smem = 2 * (size_t)ba.job[0].t.T * (ba.job[0].t.T + 1) * sizeof(float);
+    const size_t smem = warps_smem<W>();
     cudaError_t e = cudaFuncSetAttribute(grid_batch_kernel<W>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1015,6 +1388,7 @@ extern "C" rick_status rick_grid_sparse_batch(rick_plan *const *plans, void *con
         a.accumulate = 0;
         a.touched = NULL;
         a.nzero = 0;
+        set_sub_args(a, p, w);
         a.mcslot = NULL;
         a.mcacc = NULL;
         tiles_max = max(tiles_max, (int)a.t.ntiles);
