@@ -283,15 +283,27 @@ static __device__ __forceinline__ void load_sel(float2 (&x)[16], const float2 *s
 // Classes of threads whose selectors are tabled per CTA (P / T for T >= 16).
 #define RICK_FFT_SEL_CLASSES 32
 
+// Row-pass CTAs: RPR rows of P threads each at a time, BATCH times.  One batch and
+// 64 registers a thread leave room for 32 warps an SM, whose loads, transforms and
+// write-out then overlap (LOFAR-like 4096^2, 16 planes: 0.55 ms with one CTA of two
+// batches per SM); at n = 8192, where a batch is one row, a second fills the
+// sectors of the transposed store.
+template <int N>
+struct RowShape {
+    static constexpr int P = N / 16, NT = P <= 64 ? 256 : 512, RPR = NT / P;
+    static constexpr int BATCH = RPR == 1 ? 2 : 1, ROWS = RPR * BATCH;
+    static constexpr int PER_SM = BATCH == 1 ? 1024 / NT : 1;
+};
+
 // Layout of the row transforms in the work buffer, per plane k (plane stride
 // m n; the image side m is even): transposed, column p's n values contiguous
-// ([p][v]); or, where a row-pass block holds only two rows (n = 8192), in
+// ([p][v]); or, where a row-pass block holds only two rows (n = 4096, 8192), in
 // interleaved column pairs ([p/2][v][p%2]), so that the block's write-out fills
 // whole 32-byte sectors (two rows of two columns) and the column pass reads
 // every second point.
 template <int N>
 struct WorkPairs {
-    static constexpr bool ON = 1024 / (N / 16) < 4;
+    static constexpr bool ON = RowShape<N>::ROWS < 4;
     static constexpr int VS = ON ? 2 : 1;  // element stride of a column
 };
 
@@ -342,14 +354,15 @@ __global__ void __launch_bounds__(256) fft_rowflags_kernel(FftArgs a)
     }
 }
 
-// Pass 1: ROWS = 1024 / P rows per CTA, transformed in two batches by 512
-// threads (a thread's 16 points and twiddles then stay in registers), staged in
-// shared memory and written out transposed.  Persistent over (plane, block of
-// ROWS rows); blocks whose tile-rows hold no records are skipped.
+// Pass 1: ROWS rows per CTA (RowShape), staged in shared memory and written out
+// transposed.  Persistent over (plane, block of ROWS rows); blocks whose tile-rows
+// hold no records are skipped.
 template <int LOGN>
-__global__ void __launch_bounds__(512, 1) fft_rows_kernel(FftArgs a)
+__global__ void __launch_bounds__(RowShape<(1 << LOGN)>::NT, RowShape<(1 << LOGN)>::PER_SM)
+    fft_rows_kernel(FftArgs a)
 {
-    constexpr int N = 1 << LOGN, P = N / 16, ROWS = 1024 / P, RPR = 512 / P;
+    using S = RowShape<(1 << LOGN)>;
+    constexpr int N = 1 << LOGN, P = S::P, ROWS = S::ROWS, RPR = S::RPR;
     constexpr int ROT = ROWS >= 16 ? 1 : 16 / ROWS;
     constexpr int L = XLen<N>::L;
     extern __shared__ float2 sx[];  // exchange arrays (row stride L); staging at row stride N
@@ -380,7 +393,7 @@ __global__ void __launch_bounds__(512, 1) fft_rows_kernel(FftArgs a)
         }
         __syncthreads();
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < S::BATCH; ++h) {
             // the rows of batch h use their own exchange areas; the staged rows
             // of batch 0 are not touched by batch 1
             const int c = threadIdx.x / P + h * RPR, v = v0 + c;
@@ -840,13 +853,14 @@ template <int LOGN>
 static cudaError_t launch_fft_wc(const FftArgs &a, int num_sms, cudaStream_t st)
 {
     using S = ColShape<LOGN>;
-    const size_t rows_smem = sizeof(float2) * (1024 / S::P) * XLen<(1 << LOGN)>::L;
+    using RS = RowShape<(1 << LOGN)>;
+    const size_t rows_smem = sizeof(float2) * RS::ROWS * XLen<(1 << LOGN)>::L;
     cudaError_t e = fft_smem_attrs(fft_rows_kernel<LOGN>, rows_smem);
     if (e != cudaSuccess) return e;
     e = fft_smem_attrs(fft_cols_kernel<LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    const int items = a.n_w * (a.n / (1024 / S::P));
-    fft_rows_kernel<LOGN><<<(unsigned)min(items, num_sms), 512, rows_smem, st>>>(a);
+    const int items = a.n_w * (a.n / RS::ROWS);
+    fft_rows_kernel<LOGN><<<(unsigned)min(items, num_sms * RS::PER_SM), RS::NT, rows_smem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int m = a.wc.m;
