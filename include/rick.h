@@ -315,6 +315,25 @@ rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const double *uvw_d
 rick_status rick_bin_values(rick_plan *plan, const void *vis_dev, const float *weight_dev,
                             void *ws_dev, rick_bin_stats *stats_dev, void *stream);
 
+/* chi^2 = sum_m w_m |vis_m - model_m|^2 over n_vis visibilities, and the residuals
+ * vis - model in place of the model.  The sum is taken in FP64, in an order that
+ * depends on n_vis alone.
+ *   vis_dev, weight_dev: complex64 and float32 [n_vis] (weight not NULL)
+ *   model_dev:           complex64 [n_vis], overwritten with the residuals
+ *   partials_dev:        scratch of RICK_CHI2_PARTIALS float64
+ *   chi2_dev:            float32, the sum */
+#define RICK_CHI2_PARTIALS 1024
+rick_status rick_chi2_residuals(rick_plan *plan, int64_t n_vis, const void *vis_dev,
+                                const float *weight_dev, void *model_dev, double *partials_dev,
+                                float *chi2_dev, void *stream);
+
+/* rick_bin_values with the gradient of that chi^2 in the model visibilities, times
+ * *grad_dev (float32 on the device): the record values become
+ * -(*grad w)(2 r) of the residuals r; the weight sum is that of unit weights. */
+rick_status rick_bin_residuals(rick_plan *plan, const void *resid_dev, const float *weight_dev,
+                               const float *grad_dev, void *ws_dev, rick_bin_stats *stats_dev,
+                               void *stream);
+
 /* Gridding (Eq. 3): planes[k][a_y + jy][a_x + jx] +=
  * vis w G(jx - h - fx) G(jy - h - fy) for every record, with the
  * checkerboard (-1)^(i+j) of the centred FFT folded in.  Every element of

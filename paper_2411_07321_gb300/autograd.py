@@ -21,6 +21,7 @@ differentiable with respect to the image pixels.
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 
 from .imager import IMAGE_FLAGS, PREDICT_FLAGS, Imager
 
@@ -55,6 +56,33 @@ class DegridFn(torch.autograd.Function):
         return g, None, None
 
 
+class Chi2Fn(torch.autograd.Function):
+    """image -> sum w |V_obs - D x|^2 with the residuals formed, summed and binned for
+    the backward pass by the library."""
+
+    @staticmethod
+    def forward(ctx, image: torch.Tensor, imager: Imager, vis_obs: torch.Tensor,
+                weight: torch.Tensor, flags: int = PREDICT_FLAGS):
+        r = imager.adjoint(image.detach().contiguous(), None, flags)
+        loss = imager.chi2_residuals(vis_obs, weight, r)
+        ctx.save_for_backward(r, weight)
+        ctx.imager, ctx.flags = imager, flags
+        return loss
+
+    @staticmethod
+    def backward(ctx, grad_loss: torch.Tensor):
+        r, weight = ctx.saved_tensors
+        ctx.imager.bin_residuals(r, weight, grad_loss.detach().float().contiguous())
+        return ctx.imager.image_from_binned(ctx.flags), None, None, None, None
+
+
+def _plain(t, dtype, shape, device) -> bool:
+    """A tensor the library can take as it is, and that asks for no gradient."""
+    return (type(t) is torch.Tensor and t.dtype == dtype and tuple(t.shape) == shape
+            and t.device == device and t.is_contiguous() and not t.requires_grad
+            and not t.is_conj() and not t.is_neg())
+
+
 def grid_image(vis, imager, weight=None, flags=IMAGE_FLAGS):
     """Differentiable w-stacked image of ``vis`` through ``imager``'s binning."""
     return GridFn.apply(vis, imager, weight, flags)
@@ -66,6 +94,14 @@ def predict(image, imager, flags=PREDICT_FLAGS):
 
 
 def chi2(image, imager, vis_obs, weight):
-    """chi^2 = sum_m w_m |V_obs,m - (D x)_m|^2, differentiable in the image x."""
+    """chi^2 = sum_m w_m |V_obs,m - (D x)_m|^2, differentiable in the image x (and, as
+    torch operations on the model visibilities, in vis_obs and weight)."""
+    n = (imager.n_vis,)
+    if (n[0] > 0 and forward_ad._current_level < 0  # no forward-mode tangents
+            and type(image) is torch.Tensor and image.dtype == torch.float32
+            and not image.is_neg()
+            and _plain(vis_obs, torch.complex64, n, imager.device)
+            and _plain(weight, torch.float32, n, imager.device)):
+        return Chi2Fn.apply(image, imager, vis_obs, weight)
     r = vis_obs - predict(image, imager)
     return (weight * (r.real ** 2 + r.imag ** 2)).sum()

@@ -122,6 +122,29 @@ class Imager:
         R.rick_bin_values(self.plan, vis.data_ptr(), _ptr(weight), self.ws.data_ptr(),
                           self.stats_buf.data_ptr(), self._stream())
 
+    def chi2_residuals(self, vis: torch.Tensor, weight: torch.Tensor,
+                       model: torch.Tensor) -> torch.Tensor:
+        """chi^2 = sum w |vis - model|^2 (a float32 scalar on the device); the model
+        is overwritten with the residuals vis - model."""
+        n = model.shape[0]
+        self._check(vis, torch.complex64, (n,), "vis")
+        self._check(weight, torch.float32, (n,), "weight")
+        self._check(model, torch.complex64, (n,), "model")
+        part = torch.empty(R.RICK_CHI2_PARTIALS, dtype=torch.float64, device=self.device)
+        out = torch.empty((), dtype=torch.float32, device=self.device)
+        R.rick_chi2_residuals(self.plan, n, vis.data_ptr(), weight.data_ptr(), model.data_ptr(),
+                              part.data_ptr(), out.data_ptr(), self._stream())
+        return out
+
+    def bin_residuals(self, resid: torch.Tensor, weight: torch.Tensor, grad: torch.Tensor):
+        """The records' values become the gradient of that chi^2 in the model, times
+        ``grad`` (a float32 scalar on the device)."""
+        self._check(resid, torch.complex64, (self.n_vis,), "resid")
+        self._check(weight, torch.float32, (self.n_vis,), "weight")
+        self._check(grad, torch.float32, (), "grad")
+        R.rick_bin_residuals(self.plan, resid.data_ptr(), weight.data_ptr(), grad.data_ptr(),
+                             self.ws.data_ptr(), self.stats_buf.data_ptr(), self._stream())
+
     def density_weights(self, scheme: str = "briggs", robust: float = 0.0,
                         weight: torch.Tensor | None = None) -> torch.Tensor:
         """Uniform or Briggs-robust imaging weights (float32, input order) from the

@@ -70,7 +70,7 @@ EXPORTS = ["rick_status_string", "rick_plan_create", "rick_plan_destroy", "rick_
            "rick_bin_rows", "rick_image_host_rows", "rick_grid_sparse", "rick_fft_wcorrect_bytes",
            "rick_fft_wcorrect", "rick_wspread_fft", "rick_fused_work_bytes",
            "rick_probe_throughput", "rick_plan_set_wait_limit", "rick_plan_set_planes",
-           "rick_grid_sparse_batch"]
+           "rick_grid_sparse_batch", "rick_chi2_residuals", "rick_bin_residuals"]
 
 
 def _load():
@@ -99,6 +99,8 @@ def _load():
         "rick_bin": [vp, i64, vp, vp, vp, vp, sz, vp, vp],
         "rick_bin_noalloc": [vp, i64, vp, vp, vp, vp, sz, vp, vp],
         "rick_bin_values": [vp, vp, vp, vp, vp, vp],
+        "rick_chi2_residuals": [vp, i64, vp, vp, vp, vp, vp, vp],
+        "rick_bin_residuals": [vp, vp, vp, vp, vp, vp, vp],
         "rick_grid": [vp, vp, vp, vp],
         "rick_grid_accumulate": [vp, vp, vp, vp],
         "rick_grid_sparse": [vp, vp, vp, vp],
@@ -294,6 +296,19 @@ def rick_density_weights(plan, n_vis, weight, ws, scheme, robust, scratch, scrat
 def rick_bin_values(plan, vis, weight, ws, stats, stream) -> None:
     _check("rick_bin_values", _L.rick_bin_values(plan, vis, weight or None, ws, stats or None,
                                                  stream or None))
+
+
+RICK_CHI2_PARTIALS = 1024
+
+
+def rick_chi2_residuals(plan, n_vis, vis, weight, model, partials, chi2, stream) -> None:
+    _check("rick_chi2_residuals", _L.rick_chi2_residuals(plan, n_vis, vis, weight, model, partials,
+                                                         chi2, stream or None))
+
+
+def rick_bin_residuals(plan, resid, weight, grad, ws, stats, stream) -> None:
+    _check("rick_bin_residuals", _L.rick_bin_residuals(plan, resid, weight, grad, ws,
+                                                       stats or None, stream or None))
 
 
 def rick_grid(plan, ws, planes, stream) -> None:
