@@ -7,7 +7,7 @@
 // Passes, all stream-ordered:
 //   1. w range: min / max of the finite w as order-preserving integer keys
 //      (exact, deterministic), unless the range is given;
-//   2. setup: plane width, the plane boundaries as keys, plane centres;
+//   2. (its last block) plane width, the plane boundaries as keys, plane centres;
 //   3. key: per visibility two FP64 FMAs give the grid coordinates, everything
 //      else (floor, rounding, fraction, plane search) is integer work on the
 //      bit patterns -- GB300 runs FP64 at a small fraction of FP32;
@@ -86,33 +86,77 @@ static cudaError_t scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32
 // ------------------------------------------------------------------------
 // Pass 1: w range
 
+// Plane geometry (n_w <= 1024) from the range keys, by the threads of one block.
+__device__ __forceinline__ void plane_setup(WsHeader *hdr, uint64_t lo_key, uint64_t hi_key,
+                                            unsigned long long *bkey, float4 *wplane, int n_w)
+{
+    double wmin, wmax;
+    if (lo_key == ~0ull) {  // no finite w at all
+        wmin = wmax = 0.0;
+    } else {
+        wmin = rick_dunkey(lo_key);
+        wmax = rick_dunkey(hi_key);
+    }
+    const double dw = (wmax - wmin) / n_w;
+    if (threadIdx.x == 0) {
+        hdr->dw = dw;
+        hdr->stats.w_min = wmin;
+        hdr->stats.w_max = wmax;
+    }
+    for (int j = threadIdx.x; j <= n_w; j += blockDim.x) {
+        if (j >= 1 && j < n_w) bkey[j - 1] = rick_dkey(fma((double)j, dw, wmin));
+        // the entry after the last plane: the plane spacing, for the phase step
+        const double wk = j == n_w ? dw : dw == 0.0 ? wmin : fma(j + 0.5, dw, wmin);
+        const ff f = ff_from_double(wk);
+        wplane[j] = make_float4(f.hi, f.lo, (float)wk, 0.0f);
+    }
+}
+
+// The header, the zeroed histogram and, where no pass over the w has to find the
+// range (given, or nothing to look at), the planes.
 // range_src (optional): a header whose w-range keys stand in for a given
 // range (the exact range of a larger set, found by an earlier pass).
 // n_vis: records (inputs, or twice the inputs with the Hermitian mirror).
-__global__ void bin_init_kernel(WsHeader *hdr, uint64_t n_vis, uint32_t chunk_cap, int given,
-                                uint64_t wmin_key, uint64_t wmax_key, uint32_t n_key_blocks,
-                                const WsHeader *range_src, uint64_t n_src, int mirror,
-                                uint32_t sub_cap)
+__global__ void __launch_bounds__(256) bin_init_kernel(WsPtrs w, uint64_t n_vis, uint32_t chunk_cap,
+                                                       int given, uint64_t wmin_key,
+                                                       uint64_t wmax_key, uint32_t n_key_blocks,
+                                                       const WsHeader *range_src, uint64_t n_src,
+                                                       int mirror, uint32_t sub_cap, int64_t nhist,
+                                                       int n_w)
 {
-    hdr->sub_cap = sub_cap;
-    hdr->n_items = 0;
-    hdr->n_groups = 0;
-    hdr->n_vis = n_vis;
-    hdr->n_src = n_src;
-    hdr->mirror = (uint32_t)mirror;
-    hdr->fault = 0;
-    hdr->drop_uv = 0;
-    hdr->drop_w = 0;
-    hdr->chunk_cap = chunk_cap;
-    hdr->n_key_blocks = n_key_blocks;
+    const int64_t n4 = nhist / 4, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = i0; i < n4; i += (int64_t)gridDim.x * blockDim.x)
+        ((uint4 *)w.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x < nhist - 4 * n4) w.hist[4 * n4 + threadIdx.x] = 0;
     if (range_src) {
         given = 1;
         wmin_key = range_src->wmin_key;
         wmax_key = range_src->wmax_key;
     }
-    hdr->range_given = given;
-    hdr->wmin_key = given ? wmin_key : ~0ull;
-    hdr->wmax_key = given ? wmax_key : 0ull;
+    if (!given) {
+        wmin_key = ~0ull;
+        wmax_key = 0ull;
+    }
+    WsHeader *hdr = w.hdr;
+    if (threadIdx.x == 0) {
+        hdr->sub_cap = sub_cap;
+        hdr->n_items = 0;
+        hdr->n_groups = 0;
+        hdr->n_vis = n_vis;
+        hdr->n_src = n_src;
+        hdr->mirror = (uint32_t)mirror;
+        hdr->fault = 0;
+        hdr->drop_uv = 0;
+        hdr->drop_w = 0;
+        hdr->chunk_cap = chunk_cap;
+        hdr->n_key_blocks = n_key_blocks;
+        hdr->range_done = 0;
+        hdr->range_given = given;
+        hdr->wmin_key = wmin_key;
+        hdr->wmax_key = wmax_key;
+    }
+    if (given || n_vis == 0) plane_setup(hdr, wmin_key, wmax_key, w.bkey, w.wplane, n_w);
 }
 
 // Launch the w-range reduction of visibilities [0, n) into hdr's range keys.
@@ -136,9 +180,11 @@ __device__ __forceinline__ void wrange_fold(double w, uint64_t &lo, uint64_t &hi
 // row's extremes are its products with the smallest and the largest factor
 // (unless one of those overflows, when every channel is folded).
 // MIRROR: the mirrored visibilities' -w are folded in too.
+// With bkey, the block that ends last turns the range into the planes.
 template <bool MIRROR>
 __global__ void wrange_kernel(const double *uvw, int64_t n, WsHeader *hdr, int n_chan,
-                              const double *scale)
+                              const double *scale, unsigned long long *bkey, float4 *wplane,
+                              int n_w)
 {
     __shared__ double s_min[32], s_max[32];
     __shared__ int s_ok[32];
@@ -200,39 +246,23 @@ __global__ void wrange_kernel(const double *uvw, int64_t n, WsHeader *hdr, int n
         if (lo != ~0ull) atomicMin(&hdr->wmin_key, (unsigned long long)lo);
         if (hi != 0ull) atomicMax(&hdr->wmax_key, (unsigned long long)hi);
     }
+    if (!bkey) return;
+    __shared__ bool s_last;
+    __threadfence();  // this thread's minima and maxima before the block's count
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&hdr->range_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    plane_setup(hdr, *(volatile unsigned long long *)&hdr->wmin_key,
+                *(volatile unsigned long long *)&hdr->wmax_key, bkey, wplane, n_w);
 }
 
 void rick_launch_wrange(const rick_plan *plan, const double *uvw, int64_t n, WsHeader *hdr,
                         cudaStream_t st, int n_chan, const double *scale)
 {
-    wrange_kernel<false><<<plan->num_sms * 4, 256, 0, st>>>(uvw, n, hdr, n_chan, scale);
-}
-
-// ------------------------------------------------------------------------
-// Pass 2: plane geometry (one thread; n_w <= 1024)
-
-__global__ void bin_setup_kernel(WsHeader *hdr, unsigned long long *bkey, float4 *wplane, int n_w)
-{
-    double wmin, wmax;
-    if (hdr->wmin_key == ~0ull) {  // no finite w at all
-        wmin = wmax = 0.0;
-    } else {
-        wmin = rick_dunkey(hdr->wmin_key);
-        wmax = rick_dunkey(hdr->wmax_key);
-    }
-    double dw = (wmax - wmin) / n_w;
-    hdr->dw = dw;
-    hdr->stats.w_min = wmin;
-    hdr->stats.w_max = wmax;
-    for (int j = 1; j < n_w; ++j) bkey[j - 1] = rick_dkey(fma((double)j, dw, wmin));
-    for (int k = 0; k < n_w; ++k) {
-        double wk = dw == 0.0 ? wmin : fma(k + 0.5, dw, wmin);
-        ff s = ff_from_double(wk);
-        wplane[k] = make_float4(s.hi, s.lo, (float)wk, 0.0f);
-    }
-    // one more entry: the plane spacing, for the phase step between planes
-    ff d = ff_from_double(dw);
-    wplane[n_w] = make_float4(d.hi, d.lo, (float)dw, 0.0f);
+    wrange_kernel<false><<<plan->num_sms * 4, 256, 0, st>>>(uvw, n, hdr, n_chan, scale, NULL, NULL,
+                                                            0);
 }
 
 // ------------------------------------------------------------------------
@@ -455,13 +485,19 @@ __global__ void __launch_bounds__(RICK_KEY_THREADS) bin_key_kernel(KeyArgs a)
 // Weight sum over the block partials in a fixed order; stats.
 // unit_weights > 0: no weights were given, and each kept visibility weighs
 // unit_weights (its number of correlations).
-__global__ void __launch_bounds__(1024) bin_finalize_kernel(WsHeader *hdr, const double *wpart,
-                                                            int nparts, int unit_weights)
+// stats_out (optional): the caller's copy of the stats.
+__device__ __forceinline__ void bin_finalize(WsHeader *hdr, const double *wpart, int nparts,
+                                             int unit_weights, rick_bin_stats *stats_out)
 {
     __shared__ double s[1024];
-    double t = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += 1024) t += wpart[i];
-    s[threadIdx.x] = t;
+    // eight sums a thread, for as many loads in flight
+    double t8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int i = threadIdx.x; i < nparts; i += 8 * 1024) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + u * 1024 < nparts) t8[u] += wpart[i + u * 1024];
+    }
+    s[threadIdx.x] = ((t8[0] + t8[1]) + (t8[2] + t8[3])) + ((t8[4] + t8[5]) + (t8[6] + t8[7]));
     __syncthreads();
     for (int o = 512; o > 0; o >>= 1) {
         if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
@@ -474,7 +510,15 @@ __global__ void __launch_bounds__(1024) bin_finalize_kernel(WsHeader *hdr, const
         hdr->stats.n_dropped_uv = (long long)hdr->drop_uv;
         hdr->stats.n_dropped_w = (long long)hdr->drop_w;
         hdr->stats.sum_weight = unit_weights ? (double)binned * unit_weights : s[0];
+        if (stats_out) *stats_out = hdr->stats;
     }
+}
+
+__global__ void __launch_bounds__(1024) bin_finalize_kernel(WsHeader *hdr, const double *wpart,
+                                                            int nparts, int unit_weights,
+                                                            rick_bin_stats *stats_out)
+{
+    bin_finalize(hdr, wpart, nparts, unit_weights, stats_out);
 }
 
 // ------------------------------------------------------------------------
@@ -617,7 +661,8 @@ __global__ void __launch_bounds__(256) bin_values_kernel(const float2 *vis, cons
 }
 
 __global__ void __launch_bounds__(1024) values_finalize_kernel(const double *wpart, int nparts,
-                                                               int unit_weights, WsHeader *hdr)
+                                                               int unit_weights, WsHeader *hdr,
+                                                               rick_bin_stats *stats_out)
 {
     __shared__ double s[1024];
     double t = 0.0;
@@ -628,8 +673,10 @@ __global__ void __launch_bounds__(1024) values_finalize_kernel(const double *wpa
         if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         hdr->stats.sum_weight = unit_weights ? (double)hdr->stats.n_binned : s[0];
+        if (stats_out) *stats_out = hdr->stats;
+    }
 }
 
 // ------------------------------------------------------------------------
@@ -842,24 +889,29 @@ static rick_status det_sort_records(rick_plan *plan, WsPtrs w, const WsLayout &L
 // edge classes) plus the records of the west, north and north-west tiles
 // whose footprints reach into t; degridding needs only the own bin.
 
-__global__ void tile_count_kernel(const uint32_t *off, uint32_t *gcnt, uint32_t *dcnt,
-                                  uint32_t ntiles, int nt, uint32_t cap)
+// Work items (grid, degrid) of tile t; none for t = ntiles.
+__device__ __forceinline__ uint2 tile_count(const uint32_t *off, uint32_t t, uint32_t ntiles, int nt,
+                                            uint32_t cap)
 {
-    uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t > ntiles) return;
-    if (t == ntiles) {
-        gcnt[t] = 0;
-        dcnt[t] = 0;
-        return;
-    }
+    if (t >= ntiles) return make_uint2(0u, 0u);
     uint32_t tx = t % nt, ty = (t / nt) % nt;
     uint32_t own = off[4 * t + 4] - off[4 * t];
     uint32_t L = own;
     if (tx > 0) L += off[4 * (t - 1) + 3] - off[4 * (t - 1) + 1];
     if (ty > 0) L += off[4 * (t - nt) + 4] - off[4 * (t - nt) + 2];
     if (tx > 0 && ty > 0) L += off[4 * (t - nt - 1) + 3] - off[4 * (t - nt - 1) + 2];
-    gcnt[t] = (L + cap - 1) / cap;  // tiles without records: no work item
-    dcnt[t] = (own + cap - 1) / cap;
+    // tiles without records: no work item
+    return make_uint2((L + cap - 1) / cap, (own + cap - 1) / cap);
+}
+
+__global__ void tile_count_kernel(const uint32_t *off, uint32_t *gcnt, uint32_t *dcnt,
+                                  uint32_t ntiles, int nt, uint32_t cap)
+{
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t > ntiles) return;
+    const uint2 c = tile_count(off, t, ntiles, nt, cap);
+    gcnt[t] = c.x;
+    dcnt[t] = c.y;
 }
 
 // Append entries (s0 + lane of the owner, first[owner] + step i) for the cnt of
@@ -895,11 +947,11 @@ __device__ __forceinline__ void append_items(uint32_t cnt, uint32_t from, uint32
 // The plain gridding kernel's work items, in no particular order: a thread per
 // subtile counts its records (its class-0 sub-bin and, in the last column and
 // row of subtiles, those of the other classes).
-__global__ void __launch_bounds__(256) sub_items_kernel(const uint32_t *suboff, uint32_t nsubtiles,
-                                                        SubShape sub, WsHeader *hdr, uint2 *items,
-                                                        uint2 *groups)
+// All lanes of a warp, s consecutive.
+__device__ __forceinline__ void sub_items(uint32_t s, const uint32_t *suboff, uint32_t nsubtiles,
+                                          const SubShape &sub, WsHeader *hdr, uint2 *items,
+                                          uint2 *groups)
 {
-    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t cnt = 0;
     if (s < nsubtiles) {
         uint32_t n = 0;
@@ -915,13 +967,145 @@ __global__ void __launch_bounds__(256) sub_items_kernel(const uint32_t *suboff, 
     append_items(cnt - ng * RICK_SUB_GROUP, ng * RICK_SUB_GROUP, 1, s0, &hdr->n_items, items);
 }
 
-static rick_status build_items(rick_plan *plan, const WsPtrs &w, const WsLayout &L, cudaStream_t st)
+__global__ void __launch_bounds__(256) sub_items_kernel(const uint32_t *suboff, uint32_t nsubtiles,
+                                                        SubShape sub, WsHeader *hdr, uint2 *items,
+                                                        uint2 *groups)
 {
+    sub_items(blockIdx.x * blockDim.x + threadIdx.x, suboff, nsubtiles, sub, hdr, items, groups);
+}
+
+// Exclusive scan of n values by one CTA of 1024 threads, eight consecutive values a
+// thread and round: put(i, sum of get(j < i)).
+template <typename Get, typename Put>
+__device__ __forceinline__ void scan_cta(int64_t n, Get get, Put put)
+{
+    __shared__ uint32_t s_warp[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t carry = 0;
+    for (int64_t b = 0; b < n; b += 8 * 1024) {
+        const int64_t i0 = b + 8 * threadIdx.x;
+        uint32_t v[8], sum = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = i0 + u < n ? get(i0 + u) : 0u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t x = v[u];
+            v[u] = sum;
+            sum += x;
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += x;
+        }
+        __syncthreads();  // the last round's totals have been read
+        if (lane == 31) s_warp[wid] = inc;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+        for (int k = 0; k < 32; ++k) {
+            const uint32_t x = s_warp[k];
+            if (k < wid) before += x;
+            total += x;
+        }
+        const uint32_t first = carry + before + inc - sum;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i0 + u < n) put(i0 + u, first + v[u]);
+        carry += total;
+    }
+}
+
+// Everything between the key pass and the scatter, and the work lists, by one CTA:
+// for grids of few sub-bins the dozen launches of the general path cost more than
+// the work (4 planes of 512^2: 31 us of GPU time and gaps against 9).
+#define RICK_SMALL_SUBS 16384
+
+struct SmallArgs {
+    WsPtrs w;
+    SubShape sub;
+    int nparts, unit_weights, nt, plain;
+    uint32_t ntiles, cap;
+    int64_t nsubs, nbins;
+    rick_bin_stats *stats_out;
+};
+
+__global__ void __launch_bounds__(1024) bin_small_kernel(SmallArgs a)
+{
+    const WsPtrs &w = a.w;
+    bin_finalize(w.hdr, w.wpart, a.nparts, a.unit_weights, a.stats_out);
+    scan_cta(a.nsubs + 1, [&](int64_t i) { return w.hist[i]; },
+             [&](int64_t i, uint32_t v) { w.suboff[i] = v; });
+    __syncthreads();
+    for (int64_t b = threadIdx.x; b <= a.nbins; b += 1024)
+        w.offsets[b] = w.suboff[(b >> 2) * a.sub.per + rick_sub_first(a.sub, (uint32_t)b & 3u)];
+    __syncthreads();
+    scan_cta((int64_t)a.ntiles + 1,
+             [&](int64_t t) { return tile_count(w.offsets, (uint32_t)t, a.ntiles, a.nt, a.cap).x; },
+             [&](int64_t t, uint32_t v) { w.gbase[t] = v; });
+    scan_cta((int64_t)a.ntiles + 1,
+             [&](int64_t t) { return tile_count(w.offsets, (uint32_t)t, a.ntiles, a.nt, a.cap).y; },
+             [&](int64_t t, uint32_t v) { w.dbase[t] = v; });
+    if (a.plain) {
+        const uint32_t ns = a.ntiles << (2 * a.sub.lq);
+        for (uint32_t s = threadIdx.x; s < ((ns + 31) & ~31u); s += 1024)
+            sub_items(s, w.suboff, ns, a.sub, w.hdr, w.items, w.groups);
+    }
+}
+
+// The first launch of a binning: header, histogram, planes of a given range.
+static rick_status launch_init(rick_plan *plan, const WsPtrs &w, const WsLayout &L, int64_t n_vis,
+                               uint32_t cap, int given, int64_t nkb, const WsHeader *range_src,
+                               int64_t n_src, int mirror, cudaStream_t st)
+{
+    const rick_params &p = plan->p;
+    const bool own = !isnan(p.w_min);
+    int64_t blocks = (L.nsubs + 1 + 4 * 1024 - 1) / (4 * 1024);
+    if (blocks > plan->num_sms * 8) blocks = plan->num_sms * 8;
+    bin_init_kernel<<<(unsigned)blocks, 256, 0, st>>>(
+        w, (uint64_t)n_vis, cap, given, own ? rick_dkey(p.w_min) : 0, own ? rick_dkey(p.w_max) : 0,
+        (uint32_t)nkb, range_src, (uint64_t)n_src, mirror, rick_sub_cap(n_vis, plan->num_sms),
+        L.nsubs + 1, p.n_w);
+    RICK_LAUNCH_CHECK(plan);
+    return RICK_OK;
+}
+
+// After the key pass: the stats and the sub-bin and bin offsets; with small also
+// the work lists.
+static rick_status launch_offsets(rick_plan *plan, const WsPtrs &w, const WsLayout &L,
+                                  const SubShape &sub, bool small, int nparts, int unit_weights,
+                                  uint32_t cap, rick_bin_stats *stats_out, cudaStream_t st)
+{
+    if (small) {
+        const SmallArgs a = {w, sub, nparts, unit_weights, plan->p.n / plan->p.tile,
+                             rick_grid_plain(&plan->p), (uint32_t)L.ntiles, cap, L.nsubs, L.nbins,
+                             stats_out};
+        bin_small_kernel<<<1, 1024, 0, st>>>(a);
+        RICK_LAUNCH_CHECK(plan);
+        return RICK_OK;
+    }
+    bin_finalize_kernel<<<1, 1024, 0, st>>>(w.hdr, w.wpart, nparts, unit_weights, stats_out);
+    RICK_LAUNCH_CHECK(plan);
+    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, L.nsubs + 1, w.scan, st, &plan->launches));
+    bin_offsets_kernel<<<(unsigned)((L.nbins + 256) / 256), 256, 0, st>>>(w.suboff, w.offsets,
+                                                                          L.nbins, sub);
+    RICK_LAUNCH_CHECK(plan);
+    return RICK_OK;
+}
+
+static rick_status launch_lists(rick_plan *plan, const WsPtrs &w, const WsLayout &L, uint32_t cap,
+                                cudaStream_t st)
+{
+    const uint32_t nt = (uint32_t)L.ntiles;
+    tile_count_kernel<<<(nt + 256) / 256, 256, 0, st>>>(w.offsets, w.gbase, w.dbase, nt,
+                                                        plan->p.n / plan->p.tile, cap);
+    RICK_LAUNCH_CHECK(plan);
+    RICK_CUDA_TRY(plan, scan_u32(w.gbase, w.gbase, L.ntiles + 1, w.scan, st, &plan->launches));
+    RICK_CUDA_TRY(plan, scan_u32(w.dbase, w.dbase, L.ntiles + 1, w.scan, st, &plan->launches));
     if (!rick_grid_plain(&plan->p)) return RICK_OK;
     const SubShape sub = rick_sub_shape(plan->p.tile);
     const uint32_t ns = (uint32_t)(L.ntiles << (2 * sub.lq));
-    sub_items_kernel<<<(ns + 255) / 256, 256, 0, st>>>(w.suboff, ns, sub, w.hdr, w.items,
-                                                     w.groups);
+    sub_items_kernel<<<(ns + 255) / 256, 256, 0, st>>>(w.suboff, ns, sub, w.hdr, w.items, w.groups);
     RICK_LAUNCH_CHECK(plan);
     return RICK_OK;
 }
@@ -973,23 +1157,19 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     }
     int given = !isnan(p.w_min) || range_src != NULL;
 
-    bin_init_kernel<<<1, 1, 0, st>>>(w.hdr, (uint64_t)n_vis, cap, given,
-                                     isnan(p.w_min) ? 0 : rick_dkey(p.w_min),
-                                     isnan(p.w_min) ? 0 : rick_dkey(p.w_max), (uint32_t)nkb,
-                                     range_src, (uint64_t)n_src, mirror,
-                                     rick_sub_cap(n_vis, plan->num_sms));
-    RICK_LAUNCH_CHECK(plan);
+    const rick_status is = launch_init(plan, w, L, n_vis, cap, given, nkb, range_src, n_src, mirror,
+                                       st);
+    if (is != RICK_OK) return is;
     if (!given && n_vis > 0) {
         int blocks = plan->num_sms * 4;
         if (mirror)
-            wrange_kernel<true><<<blocks, 256, 0, st>>>(uvw, n_src, w.hdr, n_chan, chan_scale);
+            wrange_kernel<true><<<blocks, 256, 0, st>>>(uvw, n_src, w.hdr, n_chan, chan_scale,
+                                                        w.bkey, w.wplane, p.n_w);
         else
-            wrange_kernel<false><<<blocks, 256, 0, st>>>(uvw, n_src, w.hdr, n_chan, chan_scale);
+            wrange_kernel<false><<<blocks, 256, 0, st>>>(uvw, n_src, w.hdr, n_chan, chan_scale,
+                                                         w.bkey, w.wplane, p.n_w);
         RICK_LAUNCH_CHECK(plan);
     }
-    bin_setup_kernel<<<1, 1, 0, st>>>(w.hdr, w.bkey, w.wplane, p.n_w);
-    RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, cudaMemsetAsync(w.hist, 0, 4 * (size_t)(L.nsubs + 1), st));
 
     if (n_vis > 0) {
         KeyArgs ka;
@@ -1022,13 +1202,10 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
         bin_key_kernel<<<(unsigned)nkb, RICK_KEY_THREADS, smem, st>>>(ka);
         RICK_LAUNCH_CHECK(plan);
     }
-    bin_finalize_kernel<<<1, 1024, 0, st>>>(w.hdr, w.wpart, (int)nkb, weight == NULL ? n_corr : 0);
-    RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, L.nsubs + 1, w.scan, st,
-                                 &plan->launches));
-    bin_offsets_kernel<<<(unsigned)((L.nbins + 256) / 256), 256, 0, st>>>(w.suboff, w.offsets,
-                                                                          L.nbins, sub);
-    RICK_LAUNCH_CHECK(plan);
+    const bool small = !det && L.nsubs <= RICK_SMALL_SUBS;
+    const rick_status os = launch_offsets(plan, w, L, sub, small, (int)nkb,
+                                          weight == NULL ? n_corr : 0, cap, stats_dev, st);
+    if (os != RICK_OK) return os;
     if (det) {
         rick_status ds = det_sort_records(plan, w, L, n_vis, vis, weight, n_corr,
                                           mirror ? n_src : n_vis, st);
@@ -1047,15 +1224,10 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
                 n_vis, (const float2 *)vis, weight, w, 1, n_vis, sub);
         RICK_LAUNCH_CHECK(plan);
     }
-    uint32_t nt = (uint32_t)L.ntiles;
-    tile_count_kernel<<<(nt + 256) / 256, 256, 0, st>>>(w.offsets, w.gbase, w.dbase, nt,
-                                                        p.n / p.tile, cap);
-    RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, scan_u32(w.gbase, w.gbase, L.ntiles + 1, w.scan, st, &plan->launches));
-    RICK_CUDA_TRY(plan, scan_u32(w.dbase, w.dbase, L.ntiles + 1, w.scan, st, &plan->launches));
-    {
-        const rick_status is = build_items(plan, w, L, st);
-        if (is != RICK_OK) return is;
+    const uint32_t nt = (uint32_t)L.ntiles;
+    if (!small) {
+        const rick_status ls = launch_lists(plan, w, L, cap, st);
+        if (ls != RICK_OK) return ls;
     }
     if (det) {  // slots of the tiles with several grid work items
         det_mc_flags_kernel<<<(nt + 256) / 256, 256, 0, st>>>(w.gbase, w.mcslot, nt);
@@ -1065,9 +1237,6 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
         det_mc_count_kernel<<<1, 1, 0, st>>>(w.hdr, w.mcslot, nt);
         RICK_LAUNCH_CHECK(plan);
     }
-    if (stats_dev)
-        RICK_CUDA_TRY(plan, cudaMemcpyAsync(stats_dev, &w.hdr->stats, sizeof(rick_bin_stats),
-                                            cudaMemcpyDeviceToDevice, st));
     return RICK_OK;
 }
 
@@ -1128,15 +1297,13 @@ static rick_status bin_values_impl(rick_plan *plan, const void *vis, const float
     else
         bin_values_kernel<false><<<blocks, 256, 0, st>>>((const float2 *)vis, weight, w, det, NULL);
     RICK_LAUNCH_CHECK(plan);
-    values_finalize_kernel<<<1, 1024, 0, st>>>(w.wpart, blocks, grad || !weight, w.hdr);
+    values_finalize_kernel<<<1, 1024, 0, st>>>(w.wpart, blocks, grad || !weight, w.hdr,
+                                               stats_dev);
     RICK_LAUNCH_CHECK(plan);
     if (det) {  // the fixed-point scale for the new values
         det_scale_kernel<<<1, 1, 0, st>>>(w.hdr, w.vpart, blocks);
         RICK_LAUNCH_CHECK(plan);
     }
-    if (stats_dev)
-        RICK_CUDA_TRY(plan, cudaMemcpyAsync(stats_dev, &w.hdr->stats, sizeof(rick_bin_stats),
-                                            cudaMemcpyDeviceToDevice, st));
     return RICK_OK;
 }
 
@@ -1319,20 +1486,15 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms);
     int given = !isnan(p.w_min);
 
-    // the same stages as rick_bin, in the same order
-    bin_init_kernel<<<1, 1, 0, st>>>(w.hdr, (uint64_t)n_vis, cap, given,
-                                     given ? rick_dkey(p.w_min) : 0, given ? rick_dkey(p.w_max) : 0,
-                                     (uint32_t)nkb, NULL, (uint64_t)n_vis, 0,
-                                     rick_sub_cap(n_vis, plan->num_sms));
-    RICK_LAUNCH_CHECK(plan);
+    // the same stages as rick_bin, in the same order; the array keeps the last
+    // call's contents, and the first launch zeroes the histogram
+    const rick_status is = launch_init(plan, w, L, n_vis, cap, given, nkb, NULL, n_vis, 0, st);
+    if (is != RICK_OK) return is;
     if (!given && n_vis > 0) {
-        wrange_kernel<false><<<plan->num_sms * 4, 256, 0, st>>>(uvw, n_vis, w.hdr, 0, NULL);
+        wrange_kernel<false><<<plan->num_sms * 4, 256, 0, st>>>(uvw, n_vis, w.hdr, 0, NULL, w.bkey,
+                                                                w.wplane, p.n_w);
         RICK_LAUNCH_CHECK(plan);
     }
-    bin_setup_kernel<<<1, 1, 0, st>>>(w.hdr, w.bkey, w.wplane, p.n_w);
-    RICK_LAUNCH_CHECK(plan);
-    // the array keeps the last call's contents: the histogram must start at zero
-    RICK_CUDA_TRY(plan, cudaMemsetAsync(w.hist, 0, 4 * (size_t)(L.nsubs + 1), st));
     if (n_vis > 0) {
         KeyArgs ka;
         ka.n_vis = n_vis;
@@ -1363,13 +1525,10 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
         bin_key_kernel<<<(unsigned)nkb, RICK_KEY_THREADS, smem, st>>>(ka);
         RICK_LAUNCH_CHECK(plan);
     }
-    bin_finalize_kernel<<<1, 1024, 0, st>>>(w.hdr, w.wpart, (int)nkb, weight == NULL);
-    RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, scan_u32(w.hist, w.suboff, L.nsubs + 1, w.scan, st,
-                                 &plan->launches));
-    bin_offsets_kernel<<<(unsigned)((L.nbins + 256) / 256), 256, 0, st>>>(w.suboff, w.offsets,
-                                                                          L.nbins, sub);
-    RICK_LAUNCH_CHECK(plan);
+    const bool small = L.nsubs <= RICK_SMALL_SUBS;
+    const rick_status os = launch_offsets(plan, w, L, sub, small, (int)nkb, weight == NULL, cap,
+                                          stats_dev, st);
+    if (os != RICK_OK) return os;
     if (n_vis > 0) {
         int64_t blocks = (n_vis + 256 * RICK_SCATTER_U - 1) / (256 * RICK_SCATTER_U);
         if (blocks > (int64_t)plan->num_sms * 64) blocks = (int64_t)plan->num_sms * 64;
@@ -1377,18 +1536,6 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
             n_vis, (const float2 *)vis, weight, w, 1, n_vis, sub);
         RICK_LAUNCH_CHECK(plan);
     }
-    uint32_t nt = (uint32_t)L.ntiles;
-    tile_count_kernel<<<(nt + 256) / 256, 256, 0, st>>>(w.offsets, w.gbase, w.dbase, nt,
-                                                        p.n / p.tile, cap);
-    RICK_LAUNCH_CHECK(plan);
-    RICK_CUDA_TRY(plan, scan_u32(w.gbase, w.gbase, L.ntiles + 1, w.scan, st, &plan->launches));
-    RICK_CUDA_TRY(plan, scan_u32(w.dbase, w.dbase, L.ntiles + 1, w.scan, st, &plan->launches));
-    {
-        const rick_status is = build_items(plan, w, L, st);
-        if (is != RICK_OK) return is;
-    }
-    if (stats_dev)
-        RICK_CUDA_TRY(plan, cudaMemcpyAsync(stats_dev, &w.hdr->stats, sizeof(rick_bin_stats),
-                                            cudaMemcpyDeviceToDevice, st));
+    if (!small) return launch_lists(plan, w, L, cap, st);
     return RICK_OK;
 }

@@ -118,6 +118,7 @@ struct WsHeader {
     uint32_t zero_next;                 // counter of the grid kernel's tile-clearing items
     uint32_t fault;                     // a bounded device-side wait ran out (never expected)
     uint32_t mirror;                    // records i >= n_src mirror input i - n_src
+    uint32_t range_done;                // blocks of the w-range pass that are done
     unsigned long long n_src;           // input visibilities of the last rick_bin
     // deterministic mode: tile sums in fixed point, value = integer * fx_inv
     float fx_scale, fx_inv;             // 2^k and 2^-k
