@@ -944,27 +944,25 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
         hdr->item_next = 0;
         hdr->group_next = 0;
     }
-    int lane = threadIdx.x & 31;
-    uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int T = 1 << log2T;
-    if (mcacc) {
-        for (uint32_t t = warp; t < ntiles; t += nwarps) {
-            if (base[t + 1] - base[t] <= 1) continue;
-            ulonglong2 *slot = (ulonglong2 *)(mcacc + (size_t)mcslot[t] * 2 * T * T);
-            for (int i = lane; i < T * T; i += 32) slot[i] = make_ulonglong2(0ull, 0ull);
-        }
-        return;
-    }
-    if (accumulate) return;
+    const int lane = threadIdx.x & 31, T = 1 << log2T;
+    if (!mcacc && accumulate) return;
     // a block looks at RICK_ZERO_LOOK tiles at a time, and its warps share the rows
     // of each one to clear: the tiles with records lie side by side
     for (uint32_t t0 = blockIdx.x * RICK_ZERO_LOOK; t0 < ntiles; t0 += gridDim.x * RICK_ZERO_LOOK) {
         const uint32_t tl = t0 + lane;
         unsigned m = __ballot_sync(0xffffffffu, lane < RICK_ZERO_LOOK && tl < ntiles &&
                                                     base[tl + 1] - base[tl] >= least &&
-                                                    !(touched && touched[tl]));
-        for (; m; m &= m - 1) clear_tile(planes, t0 + __ffs(m) - 1, nt, log2T, n);
+                                                    !(!mcacc && touched && touched[tl]));
+        for (; m; m &= m - 1) {
+            const uint32_t t = t0 + __ffs(m) - 1;
+            if (!mcacc) {
+                clear_tile(planes, t, nt, log2T, n);
+                continue;
+            }
+            ulonglong2 *slot = (ulonglong2 *)(mcacc + (size_t)mcslot[t] * 2 * T * T);
+            for (int i = threadIdx.x; i < T * T; i += blockDim.x)
+                slot[i] = make_ulonglong2(0ull, 0ull);
+        }
     }
 }
 
@@ -1033,7 +1031,8 @@ __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
 
 // Deterministic mode: the tiles gridded by several work items, from their
 // int64 slots into the planes (written, or added with accumulate), the
-// checkerboard (-1)^(i+j) folded in.  One warp per tile.
+// checkerboard (-1)^(i+j) folded in.  A block per tile (a warp: 61 us for the few
+// dense tiles of 2e6 visibilities).
 __global__ void __launch_bounds__(256) det_mc_convert_kernel(const uint32_t *base, uint32_t ntiles,
                                                              int nt, int log2T, int n,
                                                              float2 *planes, const WsHeader *hdr,
@@ -1042,30 +1041,33 @@ __global__ void __launch_bounds__(256) det_mc_convert_kernel(const uint32_t *bas
                                                              const unsigned long long *mcacc)
 {
     const int lane = threadIdx.x & 31, T = 1 << log2T;
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const float inv = hdr->fx_inv;
-    for (uint32_t t = warp; t < ntiles; t += nwarps) {
-        if (base[t + 1] - base[t] <= 1) continue;
-        const uint32_t tx = t % nt, ty = (t / nt) % nt, k = t / (nt * nt);
-        const unsigned long long *slot = mcacc + (size_t)mcslot[t] * 2 * T * T;
-        float2 *plane = planes + (size_t)k * n * n;
-        for (int i = lane; i < T * T; i += 32) {
-            const int row = i >> log2T, col = i & (T - 1);
-            const int gi = (int)(tx << log2T) + col, gj = (int)(ty << log2T) + row;
-            float re = __ll2float_rn((long long)slot[2 * i]) * inv;
-            float im = __ll2float_rn((long long)slot[2 * i + 1]) * inv;
-            if ((gi + gj) & 1) {
-                re = -re;
-                im = -im;
+    for (uint32_t t0 = blockIdx.x * RICK_ZERO_LOOK; t0 < ntiles; t0 += gridDim.x * RICK_ZERO_LOOK) {
+        const uint32_t tl = t0 + lane;
+        unsigned m = __ballot_sync(0xffffffffu, lane < RICK_ZERO_LOOK && tl < ntiles &&
+                                                    base[tl + 1] - base[tl] > 1);
+        for (; m; m &= m - 1) {
+            const uint32_t t = t0 + __ffs(m) - 1;
+            const uint32_t tx = t % nt, ty = (t / nt) % nt, k = t / (nt * nt);
+            const unsigned long long *slot = mcacc + (size_t)mcslot[t] * 2 * T * T;
+            float2 *plane = planes + (size_t)k * n * n;
+            for (int i = threadIdx.x; i < T * T; i += blockDim.x) {
+                const int row = i >> log2T, col = i & (T - 1);
+                const int gi = (int)(tx << log2T) + col, gj = (int)(ty << log2T) + row;
+                float re = __ll2float_rn((long long)slot[2 * i]) * inv;
+                float im = __ll2float_rn((long long)slot[2 * i + 1]) * inv;
+                if ((gi + gj) & 1) {
+                    re = -re;
+                    im = -im;
+                }
+                float2 *dst = plane + (size_t)gj * n + gi;
+                if (accumulate) {
+                    const float2 o = *dst;
+                    re += o.x;
+                    im += o.y;
+                }
+                *dst = make_float2(re, im);
             }
-            float2 *dst = plane + (size_t)gj * n + gi;
-            if (accumulate) {
-                const float2 o = *dst;
-                re += o.x;
-                im += o.y;
-            }
-            *dst = make_float2(re, im);
         }
     }
 }
