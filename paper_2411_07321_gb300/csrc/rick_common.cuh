@@ -789,7 +789,8 @@ size_t rick_fft_work_bytes(const rick_params *p);
 // binning's to those marked), kept in the work buffer.
 rick_status rick_fft_tiles_impl(rick_plan *plan, const void *ws_dev, void *work_dev,
                                 size_t work_bytes, int mode, cudaStream_t st);
-// The fused inverse FFT + w-correction of the marked tiles.
+// The fused inverse FFT + w-correction of the marked tiles (tiles -1), or after
+// marking them as rick_fft_tiles_impl's mode 0 or 1 does.
 rick_status rick_fft_wcorrect_impl(rick_plan *plan, const void *planes_dev, const void *ws_dev,
                                    void *work_dev, size_t work_bytes, float *image_dev,
-                                   uint32_t flags, cudaStream_t st);
+                                   uint32_t flags, cudaStream_t st, int tiles = -1);

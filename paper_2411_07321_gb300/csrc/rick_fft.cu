@@ -34,6 +34,8 @@
 // The adjoint (w-spreading + forward FFT, for degridding) runs the same two
 // passes in the opposite order on the same inverse transforms, by conjugation;
 // it writes only the tiles that degridding reads (see the section below).
+#include <cooperative_groups.h>
+
 #include "rick_common.cuh"
 #include "rick_wphase.cuh"
 
@@ -325,27 +327,42 @@ __global__ void __launch_bounds__(256) fft_tiles_kernel(uint8_t *tflag, const ui
     tflag[t] = mode == 2 ? (uint8_t)(tflag[t] | has) : has;
 }
 
-// Tile-rows and planes with a tile to read: one block per plane.
-__global__ void __launch_bounds__(256) fft_rowflags_kernel(FftArgs a)
+// Tile-rows and planes with a tile to read: one block per plane, a warp per
+// tile-row.  gbase (optional): the tiles are this binning's (or with all, every
+// one), and their flags are written first; else the flags are there.
+__global__ void __launch_bounds__(256) fft_rowflags_kernel(FftArgs a, const uint32_t *gbase, int all)
 {
-    const int k = blockIdx.x, nt = a.nt;
-    const uint8_t *tf = a.tflag + (size_t)k * nt * nt;
+    const int k = blockIdx.x, nt = a.nt, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint8_t *tf = a.tflag + (size_t)k * nt * nt;
+    const uint32_t *gb = gbase ? gbase + (size_t)k * nt * nt : NULL;
     __shared__ unsigned long long s_mask[2];
     if (threadIdx.x < 2) s_mask[threadIdx.x] = 0;
     __syncthreads();
     int any_plane = 0;
-    for (int ty = threadIdx.x; ty < nt; ty += blockDim.x) {
-        uint8_t any = 0;
+    for (int ty = wid; ty < nt; ty += 8) {
+        unsigned any = 0;
         unsigned long long tm[2] = {0, 0};
-        for (int x = 0; x < nt; ++x) {
-            const uint8_t f = tf[ty * nt + x];
-            any |= f;
-            if (x < RICK_FFT_MASK_TILES && f) tm[x >> 6] |= 1ull << (x & 63);
+        for (int x0 = 0; x0 < nt; x0 += 32) {
+            const int i = ty * nt + x0 + lane;
+            bool f = false;
+            if (x0 + lane < nt) {
+                if (gb) {
+                    f = all || gb[i + 1] != gb[i];
+                    tf[i] = f;
+                } else {
+                    f = tf[i];
+                }
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, f);
+            any |= b;
+            if (x0 < RICK_FFT_MASK_TILES) tm[x0 >> 6] |= (unsigned long long)b << (x0 & 63);
         }
-        a.trow[k * nt + ty] = any;
-        a.tmask[k * nt + ty] = make_ulonglong2(tm[0], tm[1]);
-        any_plane |= any;
-        if (any && ty < RICK_FFT_MASK_TILES) atomicOr(&s_mask[ty >> 6], 1ull << (ty & 63));
+        any_plane |= any != 0;
+        if (lane == 0) {
+            a.trow[k * nt + ty] = any != 0;
+            a.tmask[k * nt + ty] = make_ulonglong2(tm[0], tm[1]);
+            if (any && ty < RICK_FFT_MASK_TILES) atomicOr(&s_mask[ty >> 6], 1ull << (ty & 63));
+        }
     }
     any_plane = __syncthreads_or(any_plane);
     if (threadIdx.x == 0) {
@@ -463,7 +480,13 @@ struct ColShape {
                                    sizeof(__half) * NE;
 };
 
-template <int LOGN>
+//
+// Where the columns fill less than the GPU, a cluster of gridDim.y CTAs takes each
+// block of columns and splits the planes; every CTA sums its planes, and each then
+// adds up its share of the pixels over the cluster's shared memory, in rank order
+// (8 planes of 256^2: 24 -> 15.5 us; 4 of 512^2: 23 -> 19).  That is SPLIT; the
+// other kernel is the same without the split's registers (3 % at n = 4096).
+template <int LOGN, bool SPLIT>
 __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 ? 2 : 1)
     fft_cols_kernel(FftArgs a)
 {
@@ -516,8 +539,10 @@ __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 
     __shared__ uint16_t s_sel[RICK_PHASE_ANCHOR][RICK_FFT_SEL_CLASSES];
     const int ncls = P >> l2T;
     const bool tabled = nt <= RICK_FFT_MASK_TILES && ncls >= 1 && ncls <= RICK_FFT_SEL_CLASSES;
-    for (int k0 = 0; k0 < w.n_w; k0 += bs) {
-        const int k1 = min(k0 + bs, w.n_w);
+    const int split = SPLIT ? gridDim.y : 1, rank = SPLIT ? blockIdx.y : 0;
+    const int nper = (w.n_w + split - 1) / split, kend = min(w.n_w, (rank + 1) * nper);
+    for (int k0 = rank * nper; k0 < kend; k0 += bs) {
+        const int k1 = min(k0 + bs, kend);
         if (tabled) {
             // the previous block's reads of the table precede the barriers of
             // its transforms
@@ -574,14 +599,29 @@ __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 
                              : fmaf(h[s].x, cs, fmaf(-h[s].y, sn, g_acc[gi]));
         }
     }
-    if (!live) return;
+    if constexpr (!SPLIT) {
+        if (!live) return;
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
-        const int q = t + P * s, gi = s * NT + threadIdx.x;
-        // n = 1 + (n - 1) to FP32 rounding
-        if (q >= off && q < off + m)
+        for (int s = 0; s < 16; ++s) {
+            const int q = t + P * s, gi = s * NT + threadIdx.x;
+            // n = 1 + (n - 1) to FP32 rounding
+            if (q >= off && q < off + m)
+                w.image_out[(size_t)(q - off) * m + pc] =
+                    g_acc[gi] * pixel_scale(w, p, q, 1.0f + g_hi[gi], inv_sumw);
+        }
+    } else {
+        const auto cluster = cooperative_groups::this_cluster();
+        cluster.sync();  // every CTA's sums are complete
+        const int share = 16 / split;  // split divides 16
+        for (int s = rank * share; s < (rank + 1) * share; ++s) {
+            const int q = t + P * s, gi = s * NT + threadIdx.x;
+            if (!live || q < off || q >= off + m) continue;
+            float sum = 0.0f;
+            for (int r = 0; r < split; ++r) sum += cluster.map_shared_rank(g_acc, r)[gi];
             w.image_out[(size_t)(q - off) * m + pc] =
-                g_acc[gi] * pixel_scale(w, p, q, 1.0f + g_hi[gi], inv_sumw);
+                sum * pixel_scale(w, p, q, 1.0f + g_hi[gi], inv_sumw);
+        }
+        cluster.sync();  // no CTA leaves while its sums are read
     }
 }
 
@@ -857,15 +897,36 @@ static cudaError_t launch_fft_wc(const FftArgs &a, int num_sms, cudaStream_t st)
     const size_t rows_smem = sizeof(float2) * RS::ROWS * XLen<(1 << LOGN)>::L;
     cudaError_t e = fft_smem_attrs(fft_rows_kernel<LOGN>, rows_smem);
     if (e != cudaSuccess) return e;
-    e = fft_smem_attrs(fft_cols_kernel<LOGN>, S::SMEM);
-    if (e != cudaSuccess) return e;
     const int items = a.n_w * (a.n / RS::ROWS);
     fft_rows_kernel<LOGN><<<(unsigned)min(items, num_sms * RS::PER_SM), RS::NT, rows_smem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int m = a.wc.m;
-    fft_cols_kernel<LOGN><<<(unsigned)((m + S::COLS - 1) / S::COLS), S::NT, S::SMEM, st>>>(a);
-    return cudaGetLastError();
+    const int m = a.wc.m, ctas = (m + S::COLS - 1) / S::COLS;
+    // planes split over clusters of up to 8 CTAs while all of them are resident at once
+    // (two a SM up to n = 4096) and each keeps a plane
+    int split = 1;
+    const int room = num_sms * (S::NT <= 256 ? 2 : 1);
+    while (split < 8 && 2 * split <= a.n_w && ctas * 2 * split <= room) split *= 2;
+    const auto cols = split == 1 ? fft_cols_kernel<LOGN, false> : fft_cols_kernel<LOGN, true>;
+    e = fft_smem_attrs(cols, S::SMEM);
+    if (e != cudaSuccess) return e;
+    if (split == 1) {
+        cols<<<(unsigned)ctas, S::NT, S::SMEM, st>>>(a);
+        return cudaGetLastError();
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1;
+    attr.val.clusterDim.y = (unsigned)split;
+    attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas, (unsigned)split);
+    cfg.blockDim = dim3(S::NT);
+    cfg.dynamicSmemBytes = S::SMEM;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cols, a);
 }
 
 static bool fft_args_ok(const rick_plan *plan, const void *ws_dev, const void *work_dev,
@@ -916,7 +977,7 @@ rick_status rick_fft_tiles_impl(rick_plan *plan, const void *ws_dev, void *work_
 
 rick_status rick_fft_wcorrect_impl(rick_plan *plan, const void *planes_dev, const void *ws_dev,
                                    void *work_dev, size_t work_bytes, float *image_dev,
-                                   uint32_t flags, cudaStream_t st)
+                                   uint32_t flags, cudaStream_t st, int tiles)
 {
     if (!fft_args_ok(plan, ws_dev, work_dev, work_bytes) || !valid_flags(flags) ||
         ((uintptr_t)planes_dev & 7) || ((uintptr_t)image_dev & 3))
@@ -925,7 +986,8 @@ rick_status rick_fft_wcorrect_impl(rick_plan *plan, const void *planes_dev, cons
     FftArgs a = fft_args(plan, ws_dev, work_dev, flags);
     a.planes = (const float2 *)planes_dev;
     a.wc.image_out = image_dev;
-    fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a);
+    const WsPtrs wp = rick_ws_ptrs((void *)ws_dev, rick_ws_layout(&p, plan->max_vis));
+    fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a, tiles < 0 ? NULL : wp.gbase, tiles == 0);
     RICK_LAUNCH_CHECK(plan);
     cudaError_t err = cudaErrorInvalidValue;
     switch (p.n) {
@@ -972,13 +1034,12 @@ extern "C" rick_status rick_wspread_fft(rick_plan *plan, const float *image_dev,
         ((uintptr_t)image_dev & 3))
         return RICK_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    rick_status s = rick_fft_tiles_impl(plan, ws_dev, work_dev, work_bytes, 1, st);
-    if (s != RICK_OK) return s;
     const rick_params &p = plan->p;
     FftArgs a = fft_args(plan, ws_dev, work_dev, flags);
     a.wc.image_in = image_dev;
     a.planes_out = (float2 *)planes_dev;
-    fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a);
+    const WsPtrs wp = rick_ws_ptrs((void *)ws_dev, rick_ws_layout(&p, plan->max_vis));
+    fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a, wp.gbase, 0);
     RICK_LAUNCH_CHECK(plan);
     cudaError_t err = cudaErrorInvalidValue;
     switch (p.n) {
@@ -1014,8 +1075,6 @@ extern "C" rick_status rick_fft_wcorrect(rick_plan *plan, const void *planes_dev
         ((uintptr_t)image_dev & 3))
         return RICK_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    rick_status s = rick_fft_tiles_impl(plan, ws_dev, work_dev, work_bytes, sparse ? 1 : 0, st);
-    if (s != RICK_OK) return s;
     return rick_fft_wcorrect_impl(plan, planes_dev, ws_dev, work_dev, work_bytes, image_dev, flags,
-                                  st);
+                                  st, sparse ? 1 : 0);
 }

@@ -1,8 +1,8 @@
 """The one-CTA pass between the key pass and the scatter (at most 16384 sub-bins)
 against the general launches, on either side of the line: offsets, work lists (by the
 planes they give) and the stats.  Corners are whole numbers and must agree exactly; the
-planes of the compensated kernel, which goes by the tile lists, are within 1e-6 of the
-plain kernel's largest cell (32 roundings of 2^-24 in about thirty terms a cell)."""
+planes of the compensated kernel, which goes by the tile lists, are within 2e-6 of the
+plain kernel."""
 import numpy as np
 import pytest
 
