@@ -738,19 +738,32 @@ __global__ void __launch_bounds__(AdjColShape<LOGN>::NT, AdjColShape<LOGN>::NT <
     }
 }
 
-// Pass B: ROWS = 1024 / P rows per CTA gathered from the transposed pass-A
-// output (lanes take consecutive rows of consecutive columns: whole 32-byte
-// sectors), staged in shared memory, transformed in two batches by 512 threads
-// (exchange arrays after the staged rows), conjugated and written to the
-// tiles with records.  Persistent over (plane, block of ROWS rows).
+// Pass B: ROWS rows per CTA gathered from the transposed pass-A output (lanes take
+// consecutive rows of consecutive columns: whole 32-byte sectors, so four rows at
+// least), staged in shared memory, transformed, conjugated and written to the tiles
+// with records.  Persistent over (plane, block of ROWS rows).  In one batch the
+// exchange arrays take the staged rows' place, and two CTAs of 64 registers a thread
+// share an SM; n = 4096 and 8192 need two batches for four (two) rows, with the
+// exchange arrays after the staged rows.
+template <int N>
+struct AdjRowShape {
+    static constexpr int P = N / 16, NT = P <= 64 ? 256 : 512, RPR = NT / P;
+    static constexpr int BATCH = RPR < 4 ? 2 : 1, ROWS = RPR * BATCH;
+    static constexpr int PER_SM = BATCH == 1 ? 1024 / NT : 1;
+    static constexpr size_t SMEM = sizeof(float2) * (BATCH == 1 ? RPR * XLen<N>::L
+                                                                : ROWS * N + RPR * XLen<N>::L);
+};
+
 template <int LOGN>
-__global__ void __launch_bounds__(512, 1) fft_rows_adj_kernel(FftArgs a)
+__global__ void __launch_bounds__(AdjRowShape<(1 << LOGN)>::NT, AdjRowShape<(1 << LOGN)>::PER_SM)
+    fft_rows_adj_kernel(FftArgs a)
 {
-    constexpr int N = 1 << LOGN, P = N / 16, ROWS = 1024 / P, RPR = 512 / P;
+    using S = AdjRowShape<(1 << LOGN)>;
+    constexpr int N = 1 << LOGN, P = S::P, ROWS = S::ROWS, RPR = S::RPR;
     constexpr int ROT = ROWS >= 16 ? 1 : 16 / ROWS;
     constexpr int L = XLen<N>::L;
     extern __shared__ float2 gx[];   // staged rows (row stride N)
-    float2 *xx = gx + ROWS * N;      // exchange arrays (row stride L)
+    float2 *xx = S::BATCH == 1 ? gx : gx + ROWS * N;  // exchange arrays (row stride L)
     __shared__ uint8_t s_tf[1024];
     const int t = threadIdx.x % P;
     const int nt = a.nt, l2T = a.log2T, m = a.wc.m, off = a.wc.off;
@@ -778,13 +791,14 @@ __global__ void __launch_bounds__(512, 1) fft_rows_adj_kernel(FftArgs a)
         }
         __syncthreads();
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < S::BATCH; ++h) {
             const int c = threadIdx.x / P + h * RPR, v = v0 + c;
             float2 x[16];
 #pragma unroll
             for (int s = 0; s < 16; ++s) {
                 x[s] = gx[swz(c * N + t + P * s) ^ ((c * ROT) & 15)];
             }
+            if (S::BATCH == 1) __syncthreads();  // the exchange overwrites the staged rows
             fft_inv<LOGN>(x, t, (threadIdx.x / P) * L, xx, a.tw);
             float2 *row = a.planes_out + ((size_t)k * N + v) * N;
             if (nt <= RICK_FFT_MASK_TILES) {
@@ -1007,19 +1021,19 @@ template <int LOGN>
 static cudaError_t launch_wspread_fft(const FftArgs &a, int num_sms, cudaStream_t st)
 {
     using S = AdjColShape<LOGN>;
-    constexpr int N = 1 << LOGN, P = N / 16, ROWS = 1024 / P, RPR = 512 / P;
-    const size_t rows_smem = sizeof(float2) * (ROWS * N + RPR * XLen<N>::L);
+    constexpr int N = 1 << LOGN;
+    using RS = AdjRowShape<N>;
     cudaError_t e = fft_smem_attrs(fft_cols_adj_kernel<LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(fft_rows_adj_kernel<LOGN>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS::SMEM);
     if (e != cudaSuccess) return e;
     const int m = a.wc.m;
     fft_cols_adj_kernel<LOGN><<<(unsigned)((m + S::COLS - 1) / S::COLS), S::NT, S::SMEM, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int items = a.n_w * (N / ROWS);
-    fft_rows_adj_kernel<LOGN><<<(unsigned)min(items, num_sms), 512, rows_smem, st>>>(a);
+    const int items = a.n_w * (N / RS::ROWS);
+    fft_rows_adj_kernel<LOGN><<<(unsigned)min(items, num_sms * RS::PER_SM), RS::NT, RS::SMEM, st>>>(a);
     return cudaGetLastError();
 }
 
