@@ -1157,7 +1157,7 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     const SubShape sub = rick_sub_shape(p.tile);
     cudaStream_t st = (cudaStream_t)stream;
     const bool det = (p.options & RICK_OPT_DETERMINISTIC) != 0;
-    uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms);
+    uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms, rick_grid_plain(&p));
     if (det) {
         // enough records per work item that the tiles with several items fit
         // the workspace's slots (a record is visited by at most four tiles)
@@ -1494,7 +1494,7 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     w.scan = (uint32_t *)(scratch + NOALLOC_SCAN);
     w.wpart = (double *)(scratch + NOALLOC_WPART);
     cudaStream_t st = (cudaStream_t)stream;
-    uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms);
+    uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms, rick_grid_plain(&p));
     int given = !isnan(p.w_min);
 
     // the same stages as rick_bin, in the same order; the array keeps the last

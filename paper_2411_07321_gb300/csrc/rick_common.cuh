@@ -382,12 +382,17 @@ static inline bool rick_grid_plain(const rick_params *p)
 // Records per work item of the tile kernels for a binning of n_vis
 // visibilities: about 64 items per SM in total (16 per resident CTA: short
 // items balance the skewed tiles of a centrally concentrated uv coverage), at
-// least 1024.  Set by the binning in the workspace header, where the tile
+// least 1024.  Where only degridding goes by tiles (plain: the gridding takes
+// subtiles), at least about 8 per SM and up to 4096: every item stages a tile of
+// its plane (1e7 visibilities, items of 1028 / 2056 / 4096: 251 / 206 / 197 us;
+// 3e6: 104 / 87 / 87).  Set by the binning in the workspace header, where the tile
 // kernels read it.
-static inline uint32_t rick_chunk_cap(int64_t n_vis, int num_sms)
+static inline uint32_t rick_chunk_cap(int64_t n_vis, int num_sms, bool plain)
 {
     int64_t c = (n_vis + (int64_t)num_sms * 64 - 1) / ((int64_t)num_sms * 64);
-    if (c < 1024) c = 1024;
+    int64_t least = plain ? n_vis / ((int64_t)num_sms * 8) : 1024;
+    least = least < 1024 ? 1024 : least > 4096 ? 4096 : least;
+    if (c < least) c = least;
     c = (c + 255) & ~(int64_t)255;
     if (c > (1 << 30)) c = 1 << 30;
     return (uint32_t)c;
