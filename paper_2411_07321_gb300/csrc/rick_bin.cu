@@ -258,6 +258,14 @@ __global__ void wrange_kernel(const double *uvw, int64_t n, WsHeader *hdr, int n
                 *(volatile unsigned long long *)&hdr->wmax_key, bkey, wplane, n_w);
 }
 
+// Blocks of the w-range pass: four uvw rows a thread for the small sets, whose
+// blocks are otherwise mostly atomics.
+static int wrange_blocks(const rick_plan *plan, int64_t units)
+{
+    const int64_t b = (units + 1023) / 1024;
+    return (int)(b < 1 ? 1 : b < plan->num_sms * 4 ? b : plan->num_sms * 4);
+}
+
 void rick_launch_wrange(const rick_plan *plan, const double *uvw, int64_t n, WsHeader *hdr,
                         cudaStream_t st, int n_chan, const double *scale)
 {
@@ -290,27 +298,6 @@ struct KeyArgs {
 static inline size_t key_pass_smem(int n_w)
 {
     return 28 * (size_t)(RICK_KEY_THREADS * RICK_KEY_ITEMS) + 8 * (size_t)(n_w > 1 ? n_w - 1 : 1);
-}
-
-// Lanes that start a run of equal keys (lane 0, or a key unlike the previous
-// lane's), as a warp ballot.
-__device__ __forceinline__ unsigned run_starts(uint32_t key, int lane)
-{
-    const uint32_t prev = __shfl_up_sync(FULL, key, 1);
-    return __ballot_sync(FULL, lane == 0 || key != prev);
-}
-
-// One past the last lane of the run that starts at or before `lane`.
-__device__ __forceinline__ int run_end(unsigned starts, int lane)
-{
-    const unsigned after = lane == 31 ? 0u : starts & (0xFFFFFFFFu << (lane + 1));
-    return after ? __ffs(after) - 1 : 32;
-}
-
-// First lane of the run that holds `lane`.
-__device__ __forceinline__ int run_begin(unsigned starts, int lane)
-{
-    return 31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)));
 }
 
 __device__ __forceinline__ uint32_t plane_of(uint64_t kw, const unsigned long long *sb, int nb)
@@ -441,17 +428,19 @@ __global__ void __launch_bounds__(RICK_KEY_THREADS) bin_key_kernel(KeyArgs a)
             }
             a.ws.key[i] = key;
         }
-        // histogram: one atomic per run of equal sub-bins in consecutive lanes
-        // (consecutive inputs -- the channels of one baseline and time -- mostly
-        // share one).  The counter's old value ranks the run inside the sub-bin,
-        // so the scatter needs no atomics of its own.
-        const unsigned starts = run_starts(sid, lane);
+        // histogram: one atomic per sub-bin that the warp's 32 inputs reach.  The
+        // counter's old value ranks the inputs inside the sub-bin, so the scatter
+        // needs no atomics of its own.  (One per run of equal sub-bins in
+        // consecutive lanes sent the core of a single-channel set to a few
+        // counters nine times a warp: 4e6 visibilities, 422 -> 296 us; 5e7 of 16
+        // channels, one or two runs a warp, 624 -> 604.)
+        const unsigned peers = __match_any_sync(FULL, sid);
+        const int first = __ffs(peers) - 1;
         uint32_t base = 0;
-        if (sid != 0xFFFFFFFFu && ((starts >> lane) & 1u))
-            base = atomicAdd(&a.ws.hist[sid], (uint32_t)(run_end(starts, lane) - lane));
-        const int first = run_begin(starts, lane);
+        if (sid != 0xFFFFFFFFu && lane == first)
+            base = atomicAdd(&a.ws.hist[sid], (uint32_t)__popc(peers));
         base = __shfl_sync(FULL, base, first);
-        if (i < a.n_vis) a.ws.rank[i] = base + (uint32_t)(lane - first);
+        if (i < a.n_vis) a.ws.rank[i] = base + (uint32_t)__popc(peers & ((1u << lane) - 1u));
     }
     // deterministic block reduction of the weight sum (double-single pairs in
     // the warp: GB300 issues FP64 slowly) and of the drop counts
@@ -1172,7 +1161,7 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
                                        st);
     if (is != RICK_OK) return is;
     if (!given && n_vis > 0) {
-        int blocks = plan->num_sms * 4;
+        const int blocks = wrange_blocks(plan, n_chan > 0 ? n_src / n_chan : n_src);
         if (mirror)
             wrange_kernel<true><<<blocks, 256, 0, st>>>(uvw, n_src, w.hdr, n_chan, chan_scale,
                                                         w.bkey, w.wplane, p.n_w);
@@ -1502,8 +1491,8 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     const rick_status is = launch_init(plan, w, L, n_vis, cap, given, nkb, NULL, n_vis, 0, st);
     if (is != RICK_OK) return is;
     if (!given && n_vis > 0) {
-        wrange_kernel<false><<<plan->num_sms * 4, 256, 0, st>>>(uvw, n_vis, w.hdr, 0, NULL, w.bkey,
-                                                                w.wplane, p.n_w);
+        wrange_kernel<false><<<wrange_blocks(plan, n_vis), 256, 0, st>>>(uvw, n_vis, w.hdr, 0, NULL,
+                                                                         w.bkey, w.wplane, p.n_w);
         RICK_LAUNCH_CHECK(plan);
     }
     if (n_vis > 0) {
