@@ -949,8 +949,8 @@ __device__ __forceinline__ void append_items(uint32_t cnt, uint32_t from, uint32
 // row of subtiles, those of the other classes).
 // All lanes of a warp, s consecutive.
 __device__ __forceinline__ void sub_items(uint32_t s, const uint32_t *suboff, uint32_t nsubtiles,
-                                          const SubShape &sub, WsHeader *hdr, uint2 *items,
-                                          uint2 *groups)
+                                          const SubShape &sub, uint32_t cap, uint32_t *n_items,
+                                          uint2 *items, uint32_t *n_groups, uint2 *groups)
 {
     uint32_t cnt = 0;
     if (s < nsubtiles) {
@@ -960,18 +960,19 @@ __device__ __forceinline__ void sub_items(uint32_t s, const uint32_t *suboff, ui
             const int64_t id = rick_subtile_range(sub, s, g);
             if (id >= 0) n += suboff[id + 1] - suboff[id];
         }
-        cnt = rick_sub_chunks(n, hdr->sub_cap);
+        cnt = rick_sub_chunks(n, cap);
     }
     const uint32_t s0 = s - (threadIdx.x & 31), ng = cnt / RICK_SUB_GROUP;
-    append_items(ng, 0, RICK_SUB_GROUP, s0, &hdr->n_groups, groups);
-    append_items(cnt - ng * RICK_SUB_GROUP, ng * RICK_SUB_GROUP, 1, s0, &hdr->n_items, items);
+    append_items(ng, 0, RICK_SUB_GROUP, s0, n_groups, groups);
+    append_items(cnt - ng * RICK_SUB_GROUP, ng * RICK_SUB_GROUP, 1, s0, n_items, items);
 }
 
 __global__ void __launch_bounds__(256) sub_items_kernel(const uint32_t *suboff, uint32_t nsubtiles,
                                                         SubShape sub, WsHeader *hdr, uint2 *items,
                                                         uint2 *groups)
 {
-    sub_items(blockIdx.x * blockDim.x + threadIdx.x, suboff, nsubtiles, sub, hdr, items, groups);
+    sub_items(blockIdx.x * blockDim.x + threadIdx.x, suboff, nsubtiles, sub, hdr->sub_cap,
+              &hdr->n_items, items, &hdr->n_groups, groups);
 }
 
 // Exclusive scan of n values by one CTA of 1024 threads, eight consecutive values a
@@ -1047,9 +1048,18 @@ __global__ void __launch_bounds__(1024) bin_small_kernel(SmallArgs a)
              [&](int64_t t) { return tile_count(w.offsets, (uint32_t)t, a.ntiles, a.nt, a.cap).y; },
              [&](int64_t t, uint32_t v) { w.dbase[t] = v; });
     if (a.plain) {
-        const uint32_t ns = a.ntiles << (2 * a.sub.lq);
+        // the lists' lengths in shared memory until they are known
+        __shared__ uint32_t s_len[2];
+        if (threadIdx.x < 2) s_len[threadIdx.x] = 0;
+        __syncthreads();
+        const uint32_t ns = a.ntiles << (2 * a.sub.lq), cap = w.hdr->sub_cap;
         for (uint32_t s = threadIdx.x; s < ((ns + 31) & ~31u); s += 1024)
-            sub_items(s, w.suboff, ns, a.sub, w.hdr, w.items, w.groups);
+            sub_items(s, w.suboff, ns, a.sub, cap, &s_len[0], w.items, &s_len[1], w.groups);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            w.hdr->n_items = s_len[0];
+            w.hdr->n_groups = s_len[1];
+        }
     }
 }
 
