@@ -282,6 +282,74 @@ static __device__ __forceinline__ void load_sel(float2 (&x)[16], const float2 *s
         x[s] = ((sel >> s) & 1u) ? __ldcg(src + VS * (t + P * s)) : make_float2(0.0f, 0.0f);
 }
 
+// Opposite planes.  The image is Re sum_k F_k e^{2 pi i w_k (n - 1)}.  Where the w
+// range is symmetric about zero (a given range, or the Hermitian mirror's), plane
+// k' = n_w - 1 - k has w_k' = -w_k, and the two contribute
+// Re (F_k + conj F_k') e^{2 pi i w_k (n - 1)}: one transform, of
+// g_k[v][u] + conj g_k'[-v][-u] (indices mod n; the checkerboard is even in both).  So
+// half the planes are transformed; the middle one of an odd number is its own
+// opposite (w = 0) and goes alone.
+//
+// FOLD: the kernels for plans whose range is symmetric (the binning's decides); the
+// others are without it (its registers cost the row pass of n = 8192 7 %).  16 planes
+// of 4096^2, 32e6 visibilities in the streamed call: rows 506 -> 370 us, columns 871
+// -> 555; both sides' tile-rows are read for the half of the planes.
+template <bool FOLD>
+struct Fold {
+    int planes;  // planes to transform
+    bool on;
+    __device__ __forceinline__ int opposite(int k, int n_w) const
+    {
+        return FOLD && on && n_w - 1 - k != k ? n_w - 1 - k : -1;
+    }
+};
+
+template <bool FOLD>
+static __device__ __forceinline__ Fold<FOLD> plane_fold(const FftArgs &a)
+{
+    if (!FOLD) return {a.n_w, false};
+    const rick_bin_stats &s = a.wc.hdr->stats;
+    const bool on = a.n_w > 1 && s.w_min == -s.w_max && s.w_min < s.w_max;
+    return {on ? (a.n_w + 1) / 2 : a.n_w, on};
+}
+
+// Whether tile-row ty of plane k holds records, or a mirrored row of plane ko (if any)
+// lies in it: row v of it is row n - v of tile-row nt - 1 - ty, or for its first row
+// of tile-row nt - ty (mod nt).
+static __device__ __forceinline__ bool fold_row(const FftArgs &a, int k, int ko, int ty)
+{
+    bool any = a.trow[k * a.nt + ty] != 0;
+    if (ko >= 0)
+        any |= a.trow[ko * a.nt + a.nt - 1 - ty] != 0 ||
+               a.trow[ko * a.nt + (ty ? a.nt - ty : 0)] != 0;
+    return any;
+}
+
+// The same for every tile-row as a mask (nt <= 128).
+static __device__ __forceinline__ ulonglong2 fold_mask(const FftArgs &a, int k, int ko)
+{
+    ulonglong2 m = a.pmask[k];
+    if (ko < 0) return m;
+    const ulonglong2 o = a.pmask[ko];
+    // bits reversed within 128, then down to nt: r[ty] = o[nt - 1 - ty]
+    unsigned long long lo = __brevll(o.y), hi = __brevll(o.x);
+    const int sh = 128 - a.nt;
+    if (sh >= 64) {
+        lo = hi >> (sh - 64);
+        hi = 0;
+    } else if (sh > 0) {
+        lo = lo >> sh | hi << (64 - sh);
+        hi >>= sh;
+    }
+    m.x |= lo | lo << 1 | (o.x & 1ull);  // r, r one up, and o[0] for ty = 0
+    m.y |= hi | hi << 1 | lo >> 63;
+    // (the bit shifted past tile-row nt - 1 is o[0]'s; rows end there)
+    if (a.nt < 64) m.x &= (1ull << a.nt) - 1;
+    if (a.nt < 64) m.y = 0;
+    else if (a.nt < 128) m.y &= (1ull << (a.nt - 64)) - 1;
+    return m;
+}
+
 // Classes of threads whose selectors are tabled per CTA (P / T for T >= 16).
 #define RICK_FFT_SEL_CLASSES 32
 
@@ -371,10 +439,33 @@ __global__ void __launch_bounds__(256) fft_rowflags_kernel(FftArgs a, const uint
     }
 }
 
+// x[s] += conj g_ko[-v][-(t + P s)] where that cell's tile holds records.
+template <int P, int N>
+static __device__ __forceinline__ void add_opposite(float2 (&x)[16], const FftArgs &a, int ko, int v,
+                                                    int t)
+{
+    const int vo = (N - v) & (N - 1), l2T = a.log2T, nt = a.nt;
+    const size_t tr = (size_t)ko * nt + (vo >> l2T);
+    if (!a.trow[tr]) return;
+    const float2 *row = a.planes + ((size_t)ko * N + vo) * N;
+    const bool masks = nt <= RICK_FFT_MASK_TILES;
+    const ulonglong2 msk = masks ? a.tmask[tr] : make_ulonglong2(0ull, 0ull);
+    const uint8_t *tf = a.tflag + tr * nt;
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+        const int uo = (N - t - P * s) & (N - 1);
+        if (masks ? mask_bit(msk, uo >> l2T) : tf[uo >> l2T] != 0) {
+            const float2 g = __ldcg(row + uo);
+            x[s].x += g.x;
+            x[s].y -= g.y;
+        }
+    }
+}
+
 // Pass 1: ROWS rows per CTA (RowShape), staged in shared memory and written out
 // transposed.  Persistent over (plane, block of ROWS rows); blocks whose tile-rows
 // hold no records are skipped.
-template <int LOGN>
+template <int LOGN, bool FOLD>
 __global__ void __launch_bounds__(RowShape<(1 << LOGN)>::NT, RowShape<(1 << LOGN)>::PER_SM)
     fft_rows_kernel(FftArgs a)
 {
@@ -392,12 +483,13 @@ __global__ void __launch_bounds__(RowShape<(1 << LOGN)>::NT, RowShape<(1 << LOGN
     const int ncls = P >> l2T;
     const bool tabled = nt > 64 && nt <= RICK_FFT_MASK_TILES && ncls >= 1 &&
                         ncls <= RICK_FFT_SEL_CLASSES && ROWS <= 8 << l2T;
-    const int nvb = N / ROWS, items = a.n_w * nvb;
+    const Fold<FOLD> fold = plane_fold<FOLD>(a);
+    const int nvb = N / ROWS, items = fold.planes * nvb;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
-        const int k = item / nvb, v0 = (item - k * nvb) * ROWS;
+        const int k = item / nvb, v0 = (item - k * nvb) * ROWS, ko = fold.opposite(k, a.n_w);
         const int ty0 = v0 >> l2T, ty1 = (v0 + ROWS - 1) >> l2T;
         bool any = false;
-        for (int ty = ty0; ty <= ty1; ++ty) any |= a.trow[k * nt + ty] != 0;
+        for (int ty = ty0; ty <= ty1; ++ty) any |= fold_row(a, k, ko, ty);
         if (!any) continue;  // the same for every thread
         __syncthreads();     // the previous block's write-out has read the staging rows
         const int ntr = ty1 - ty0 + 1;
@@ -430,6 +522,7 @@ __global__ void __launch_bounds__(RowShape<(1 << LOGN)>::NT, RowShape<(1 << LOGN
                     x[s] = tf[u >> l2T] ? __ldcg(row + u) : make_float2(0.0f, 0.0f);
                 }
             }
+            if (ko >= 0) add_opposite<P, N>(x, a, ko, v, t);
             fft_inv<LOGN>(x, t, c * L, sx, a.tw);
             // stage the row (row stride N: the staged rows of batch 0 lie below
             // the exchange arrays of batch 1), XOR-swizzled and rotated per row
@@ -486,7 +579,7 @@ struct ColShape {
 // adds up its share of the pixels over the cluster's shared memory, in rank order
 // (8 planes of 256^2: 24 -> 15.5 us; 4 of 512^2: 23 -> 19).  That is SPLIT; the
 // other kernel is the same without the split's registers (3 % at n = 4096).
-template <int LOGN, bool SPLIT>
+template <int LOGN, bool SPLIT, bool FOLD>
 __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 ? 2 : 1)
     fft_cols_kernel(FftArgs a)
 {
@@ -540,7 +633,8 @@ __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 
     const int ncls = P >> l2T;
     const bool tabled = nt <= RICK_FFT_MASK_TILES && ncls >= 1 && ncls <= RICK_FFT_SEL_CLASSES;
     const int split = SPLIT ? gridDim.y : 1, rank = SPLIT ? blockIdx.y : 0;
-    const int nper = (w.n_w + split - 1) / split, kend = min(w.n_w, (rank + 1) * nper);
+    const Fold<FOLD> fold = plane_fold<FOLD>(a);
+    const int nper = (fold.planes + split - 1) / split, kend = min(fold.planes, (rank + 1) * nper);
     for (int k0 = rank * nper; k0 < kend; k0 += bs) {
         const int k1 = min(k0 + bs, kend);
         if (tabled) {
@@ -548,7 +642,8 @@ __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 
             // its transforms
             for (int i = threadIdx.x; i < (k1 - k0) * ncls; i += NT) {
                 const int r = i / ncls, c = i - r * ncls;
-                s_sel[r][c] = (uint16_t)class_sel(a.pmask[k0 + r], c, ncls);
+                s_sel[r][c] = (uint16_t)class_sel(fold_mask(a, k0 + r, fold.opposite(k0 + r, w.n_w)),
+                                                  c, ncls);
             }
             __syncthreads();
         }
@@ -556,7 +651,8 @@ __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 
 #pragma unroll
         for (int s = 0; s < 16; ++s) h[s] = make_float2(0.0f, 0.0f);
         for (int k = k1 - 1; k >= k0; --k) {
-            if (!a.pflag[k]) {  // an empty plane adds nothing: h = h D
+            const int ko = fold.opposite(k, w.n_w);
+            if (!a.pflag[k] && (ko < 0 || !a.pflag[ko])) {  // an empty plane adds nothing: h = h D
 #pragma unroll
                 for (int s = 0; s < 16; ++s) h[s] = cmul(h[s], D[s]);
                 continue;
@@ -566,15 +662,15 @@ __global__ void __launch_bounds__(ColShape<LOGN>::NT, ColShape<LOGN>::NT <= 256 
             if (tabled) {
                 load_sel<P, VS>(x, src, live ? (uint32_t)s_sel[k - k0][t >> l2T] : 0u, t);
             } else if (nt <= RICK_FFT_MASK_TILES) {  // the plane's tile-rows as a bit mask
-                const ulonglong2 msk = live ? a.pmask[k] : make_ulonglong2(0ull, 0ull);
+                const ulonglong2 msk = live ? fold_mask(a, k, ko) : make_ulonglong2(0ull, 0ull);
                 if (nt <= 64) load_masked<P, false, VS>(x, src, msk, t, l2T);
                 else load_masked<P, true, VS>(x, src, msk, t, l2T);
             } else {
-                const uint8_t *tr = a.trow + k * nt;
 #pragma unroll
                 for (int s = 0; s < 16; ++s) {
                     const int v = t + P * s;
-                    x[s] = (live && tr[v >> l2T]) ? __ldcg(src + VS * v) : make_float2(0.0f, 0.0f);
+                    x[s] = (live && fold_row(a, k, ko, v >> l2T)) ? __ldcg(src + VS * v)
+                                                                  : make_float2(0.0f, 0.0f);
                 }
             }
             fft_inv<LOGN>(x, t, cb, sx, a.tw);
@@ -904,15 +1000,16 @@ static cudaError_t fft_smem_attrs(K kernel, size_t smem)
 }
 
 template <int LOGN>
-static cudaError_t launch_fft_wc(const FftArgs &a, int num_sms, cudaStream_t st)
+static cudaError_t launch_fft_wc(const FftArgs &a, bool fold, int num_sms, cudaStream_t st)
 {
     using S = ColShape<LOGN>;
     using RS = RowShape<(1 << LOGN)>;
     const size_t rows_smem = sizeof(float2) * RS::ROWS * XLen<(1 << LOGN)>::L;
-    cudaError_t e = fft_smem_attrs(fft_rows_kernel<LOGN>, rows_smem);
+    const auto rows = fold ? fft_rows_kernel<LOGN, true> : fft_rows_kernel<LOGN, false>;
+    cudaError_t e = fft_smem_attrs(rows, rows_smem);
     if (e != cudaSuccess) return e;
     const int items = a.n_w * (a.n / RS::ROWS);
-    fft_rows_kernel<LOGN><<<(unsigned)min(items, num_sms * RS::PER_SM), RS::NT, rows_smem, st>>>(a);
+    rows<<<(unsigned)min(items, num_sms * RS::PER_SM), RS::NT, rows_smem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int m = a.wc.m, ctas = (m + S::COLS - 1) / S::COLS;
@@ -920,8 +1017,10 @@ static cudaError_t launch_fft_wc(const FftArgs &a, int num_sms, cudaStream_t st)
     // (two a SM up to n = 4096) and each keeps a plane
     int split = 1;
     const int room = num_sms * (S::NT <= 256 ? 2 : 1);
-    while (split < 8 && 2 * split <= a.n_w && ctas * 2 * split <= room) split *= 2;
-    const auto cols = split == 1 ? fft_cols_kernel<LOGN, false> : fft_cols_kernel<LOGN, true>;
+    while (!fold && split < 8 && 2 * split <= a.n_w && ctas * 2 * split <= room) split *= 2;
+    const auto cols = fold ? fft_cols_kernel<LOGN, false, true>
+                    : split == 1 ? fft_cols_kernel<LOGN, false, false>
+                                 : fft_cols_kernel<LOGN, true, false>;
     e = fft_smem_attrs(cols, S::SMEM);
     if (e != cudaSuccess) return e;
     if (split == 1) {
@@ -1003,14 +1102,18 @@ rick_status rick_fft_wcorrect_impl(rick_plan *plan, const void *planes_dev, cons
     const WsPtrs wp = rick_ws_ptrs((void *)ws_dev, rick_ws_layout(&p, plan->max_vis));
     fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a, tiles < 0 ? NULL : wp.gbase, tiles == 0);
     RICK_LAUNCH_CHECK(plan);
+    // a real image of a symmetric w range
+    const bool fold = !(flags & RICK_IMAG_PART) && p.n_w > 1 &&
+                      ((p.options & RICK_OPT_HERMITIAN_MIRROR) ||
+                       (p.w_min == -p.w_max && p.w_min < p.w_max));
     cudaError_t err = cudaErrorInvalidValue;
     switch (p.n) {
-    case 256: err = launch_fft_wc<8>(a, plan->num_sms, st); break;
-    case 512: err = launch_fft_wc<9>(a, plan->num_sms, st); break;
-    case 1024: err = launch_fft_wc<10>(a, plan->num_sms, st); break;
-    case 2048: err = launch_fft_wc<11>(a, plan->num_sms, st); break;
-    case 4096: err = launch_fft_wc<12>(a, plan->num_sms, st); break;
-    case 8192: err = launch_fft_wc<13>(a, plan->num_sms, st); break;
+    case 256: err = launch_fft_wc<8>(a, fold, plan->num_sms, st); break;
+    case 512: err = launch_fft_wc<9>(a, fold, plan->num_sms, st); break;
+    case 1024: err = launch_fft_wc<10>(a, fold, plan->num_sms, st); break;
+    case 2048: err = launch_fft_wc<11>(a, fold, plan->num_sms, st); break;
+    case 4096: err = launch_fft_wc<12>(a, fold, plan->num_sms, st); break;
+    case 8192: err = launch_fft_wc<13>(a, fold, plan->num_sms, st); break;
     }
     plan->launches += 2;
     RICK_CUDA_TRY(plan, err);
