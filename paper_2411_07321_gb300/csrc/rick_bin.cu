@@ -479,14 +479,9 @@ __device__ __forceinline__ void bin_finalize(WsHeader *hdr, const double *wpart,
                                              int unit_weights, rick_bin_stats *stats_out)
 {
     __shared__ double s[1024];
-    // eight sums a thread, for as many loads in flight
-    double t8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nparts; i += 8 * 1024) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (i + u * 1024 < nparts) t8[u] += wpart[i + u * 1024];
-    }
-    s[threadIdx.x] = ((t8[0] + t8[1]) + (t8[2] + t8[3])) + ((t8[4] + t8[5]) + (t8[6] + t8[7]));
+    double t = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += 1024) t += wpart[i];
+    s[threadIdx.x] = t;
     __syncthreads();
     for (int o = 512; o > 0; o >>= 1) {
         if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
@@ -1113,7 +1108,7 @@ static rick_status launch_lists(rick_plan *plan, const WsPtrs &w, const WsLayout
     RICK_CUDA_TRY(plan, scan_u32(w.gbase, w.gbase, L.ntiles + 1, w.scan, st, &plan->launches));
     RICK_CUDA_TRY(plan, scan_u32(w.dbase, w.dbase, L.ntiles + 1, w.scan, st, &plan->launches));
     if (!rick_grid_plain(&plan->p)) return RICK_OK;
-    const SubShape sub = rick_sub_shape(plan->p.tile);
+    const SubShape sub = rick_sub_shape(&plan->p);
     const uint32_t ns = (uint32_t)(L.ntiles << (2 * sub.lq));
     sub_items_kernel<<<(ns + 255) / 256, 256, 0, st>>>(w.suboff, ns, sub, w.hdr, w.items, w.groups);
     RICK_LAUNCH_CHECK(plan);
@@ -1153,7 +1148,7 @@ rick_status rick_bin_impl(rick_plan *plan, int64_t n_vis, const double *uvw, con
     const int64_t nkb = (n_vis + RICK_KEY_THREADS * RICK_KEY_ITEMS - 1) /
                         (RICK_KEY_THREADS * RICK_KEY_ITEMS);
     WsPtrs w = rick_ws_ptrs(ws_dev, L);
-    const SubShape sub = rick_sub_shape(p.tile);
+    const SubShape sub = rick_sub_shape(&p);
     cudaStream_t st = (cudaStream_t)stream;
     const bool det = (p.options & RICK_OPT_DETERMINISTIC) != 0;
     uint32_t cap = rick_chunk_cap(n_vis, plan->num_sms, rick_grid_plain(&p));
@@ -1486,7 +1481,7 @@ extern "C" rick_status rick_bin_noalloc(rick_plan *plan, int64_t n_vis, const do
     // outputs (records, offsets, work lists, and the keys and corner cells that
     // later calls read) in the caller's workspace, temporaries in the fixed array
     WsPtrs w = rick_ws_ptrs(ws_dev, L);
-    const SubShape sub = rick_sub_shape(p.tile);
+    const SubShape sub = rick_sub_shape(&p);
     w.rank = (uint32_t *)(scratch + NOALLOC_RANK);
     w.frac = (float2 *)(scratch + NOALLOC_FRAC);
     w.hist = (uint32_t *)(scratch + NOALLOC_HIST);

@@ -155,12 +155,22 @@ struct SubShape {
     int log2T, ls, lq, per;  // tile side, subtile side, subtiles per side (logs); sub-bins per tile
 };
 
-RICK_HD SubShape rick_sub_shape(int tile)
+// Plans gridded by the plain kernel, in subtiles (else by tiles: compensated
+// and deterministic sums).
+static inline bool rick_grid_plain(const rick_params *p)
+{
+    return p->precision == RICK_PREC_FP32 && !(p->options & RICK_OPT_DETERMINISTIC);
+}
+
+// (Plans that grid by tiles keep a bin's records as they arrive, one sub-bin a bin:
+// by subtile, neighbouring record streams add to the same cells, and the compensated
+// kernel ran 10 % slower.)
+static inline SubShape rick_sub_shape(const rick_params *p)
 {
     SubShape s;
     s.log2T = 0;
-    while ((1 << s.log2T) < tile) ++s.log2T;
-    s.ls = s.log2T < RICK_SUB_LOG ? s.log2T : RICK_SUB_LOG;
+    while ((1 << s.log2T) < p->tile) ++s.log2T;
+    s.ls = s.log2T < RICK_SUB_LOG || !rick_grid_plain(p) ? s.log2T : RICK_SUB_LOG;
     s.lq = s.log2T - s.ls;
     s.per = ((1 << s.lq) + 1) * ((1 << s.lq) + 1);
     return s;
@@ -274,7 +284,7 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
     L.nbins = 4 * L.ntiles;
     L.nkeyblocks = (n_vis + RICK_KEY_THREADS * RICK_KEY_ITEMS - 1) / (RICK_KEY_THREADS * RICK_KEY_ITEMS);
     L.ndetblocks = det ? (n_vis + RICK_DET_BLOCK - 1) / RICK_DET_BLOCK : 0;
-    const SubShape sub = rick_sub_shape(p->tile);
+    const SubShape sub = rick_sub_shape(p);
     L.nsubs = L.ntiles * sub.per;
     // work items: at most one per subtile that holds records, and one more per
     // RICK_SUB_CAP_MIN records
@@ -370,13 +380,6 @@ static inline WsPtrs rick_ws_ptrs(void *ws, const WsLayout &L)
     w.items = (uint2 *)(b + L.items);
     w.groups = (uint2 *)(b + L.groups);
     return w;
-}
-
-// Plans gridded by the plain kernel, in subtiles (else by tiles: compensated
-// and deterministic sums).
-static inline bool rick_grid_plain(const rick_params *p)
-{
-    return p->precision == RICK_PREC_FP32 && !(p->options & RICK_OPT_DETERMINISTIC);
 }
 
 // Records per work item of the tile kernels for a binning of n_vis

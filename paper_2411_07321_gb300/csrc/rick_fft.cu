@@ -395,10 +395,10 @@ __global__ void __launch_bounds__(256) fft_tiles_kernel(uint8_t *tflag, const ui
     tflag[t] = mode == 2 ? (uint8_t)(tflag[t] | has) : has;
 }
 
-// Tile-rows and planes with a tile to read: one block per plane, a warp per
-// tile-row.  gbase (optional): the tiles are this binning's (or with all, every
+// Tile-rows and planes with a tile to read: one block of 32 warps per plane, a warp
+// per tile-row at a time (with eight warps, 30 us of load latency at 128 a side).  gbase (optional): the tiles are this binning's (or with all, every
 // one), and their flags are written first; else the flags are there.
-__global__ void __launch_bounds__(256) fft_rowflags_kernel(FftArgs a, const uint32_t *gbase, int all)
+__global__ void __launch_bounds__(1024) fft_rowflags_kernel(FftArgs a, const uint32_t *gbase, int all)
 {
     const int k = blockIdx.x, nt = a.nt, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint8_t *tf = a.tflag + (size_t)k * nt * nt;
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(256) fft_rowflags_kernel(FftArgs a, const uint
     if (threadIdx.x < 2) s_mask[threadIdx.x] = 0;
     __syncthreads();
     int any_plane = 0;
-    for (int ty = wid; ty < nt; ty += 8) {
+    for (int ty = wid; ty < nt; ty += 32) {
         unsigned any = 0;
         unsigned long long tm[2] = {0, 0};
         for (int x0 = 0; x0 < nt; x0 += 32) {
@@ -1100,7 +1100,7 @@ rick_status rick_fft_wcorrect_impl(rick_plan *plan, const void *planes_dev, cons
     a.planes = (const float2 *)planes_dev;
     a.wc.image_out = image_dev;
     const WsPtrs wp = rick_ws_ptrs((void *)ws_dev, rick_ws_layout(&p, plan->max_vis));
-    fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a, tiles < 0 ? NULL : wp.gbase, tiles == 0);
+    fft_rowflags_kernel<<<p.n_w, 1024, 0, st>>>(a, tiles < 0 ? NULL : wp.gbase, tiles == 0);
     RICK_LAUNCH_CHECK(plan);
     // a real image of a symmetric w range
     const bool fold = !(flags & RICK_IMAG_PART) && p.n_w > 1 &&
@@ -1156,7 +1156,7 @@ extern "C" rick_status rick_wspread_fft(rick_plan *plan, const float *image_dev,
     a.wc.image_in = image_dev;
     a.planes_out = (float2 *)planes_dev;
     const WsPtrs wp = rick_ws_ptrs((void *)ws_dev, rick_ws_layout(&p, plan->max_vis));
-    fft_rowflags_kernel<<<p.n_w, 256, 0, st>>>(a, wp.gbase, 0);
+    fft_rowflags_kernel<<<p.n_w, 1024, 0, st>>>(a, wp.gbase, 0);
     RICK_LAUNCH_CHECK(plan);
     cudaError_t err = cudaErrorInvalidValue;
     switch (p.n) {

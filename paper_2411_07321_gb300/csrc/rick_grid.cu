@@ -155,6 +155,19 @@ __device__ __forceinline__ void warp_flush(float2 *cells, int fb, const float *a
     for (int jx = 0; jx < W; ++jx) p[jx] = make_float2(o[jx].x + ar[jx], o[jx].y + ai[jx]);
 }
 
+// The same while the other groups add theirs, two float adds a cell.
+template <int W>
+__device__ __forceinline__ void warp_flush_atomic(float2 *cells, int fb, const float *ar,
+                                                  const float *ai)
+{
+    float *p = (float *)(cells + fb);
+#pragma unroll
+    for (int jx = 0; jx < W; ++jx) {
+        atomicAdd(p + 2 * jx, ar[jx]);
+        atomicAdd(p + 2 * jx + 1, ai[jx]);
+    }
+}
+
 // The same into the 64-bit fixed-point tile: each row sum scaled by 2^k and
 // rounded to an integer, then added with integer atomics (exact, so the tile
 // does not depend on the order in which the groups flush).
@@ -543,7 +556,7 @@ __device__ __forceinline__ void zero_group(const GridArgs &a, uint32_t z)
 }
 
 // This lane's kernel segment (= its footprint row within its group).
-template <int W>
+template <int W, bool PIN = true>
 __device__ __forceinline__ void load_coef(const KernelPoly &kp, float2 *coef2)
 {
     const int seg = min((int)((threadIdx.x & 31) % StreamShape<W>::G), W - 1);
@@ -552,7 +565,7 @@ __device__ __forceinline__ void load_coef(const KernelPoly &kp, float2 *coef2)
         coef2[k] = make_float2(kp.c[seg][k], kp.c[seg][k]);
         // opaque from here on: the compiler would rather read them again in every
         // step than keep them, and a lane-indexed constant load is a replay per row
-        asm volatile("" : "+f"(coef2[k].x), "+f"(coef2[k].y));
+        if (PIN) asm volatile("" : "+f"(coef2[k].x), "+f"(coef2[k].y));
     }
 }
 
@@ -568,7 +581,7 @@ __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, 3) grid_kernel(GridArgs 
     __shared__ uint32_t s_b, s_tile, s_z;
     const uint32_t total = a.t.base[a.t.ntiles];
     float2 coef2[RICK_POLY_N];
-    load_coef<W>(a.t.kp, coef2);
+    load_coef<W, false>(a.t.kp, coef2);
     for (;;) {
         if (threadIdx.x == 0) {
             const uint32_t b = atomicAdd(&a.t.hdr->grid_next, 1u);
@@ -609,6 +622,9 @@ __device__ __forceinline__ void warp_stream(const TileArgs &ta, uint32_t r0, uin
                                             float2 *cells)
 {
     constexpr int G = StreamShape<W>::G, NGR = StreamShape<W>::NG, ST = SubCells<W>::STRIDE;
+    // Narrow kernels have eight groups a warp and more: taking turns costs more than
+    // the few compare-and-swap loops of a row.
+    constexpr bool ATOMIC = NGR > 4;
     using Ring = RecRing<W>;
     constexpr int RB = RICK_GRID_RB, NH = (Ring::SLOTS + 31) / 32;
     __shared__ __align__(16) float4 s_rrec[Ring::ON ? RICK_GRID_WARPS * 2 * Ring::SLOTS : 1];
@@ -650,6 +666,8 @@ __device__ __forceinline__ void warp_stream(const TileArgs &ta, uint32_t r0, uin
         cur = ta.rcell[r];
     }
     uint32_t cell = cur;
+    // (unrolled by two, the ring's loop gains 3.5 % at W = 9, the other loses as much)
+#pragma unroll(Ring::ON ? 2 : 1)
     for (uint32_t i = 0; i < ntrip; ++i) {
         // the next record; past the stream's end the last one again
         float4 nq;
@@ -675,13 +693,20 @@ __device__ __forceinline__ void warp_stream(const TileArgs &ta, uint32_t r0, uin
             ncell = wcel[ri];
         } else {
             r = min(r + 1, last);
-            nq = ta.rec[r];
-            ncell = ta.rcell[r];
+            nq = __ldg(ta.rec + r);
+            ncell = __ldg(ta.rcell + r);
         }
-        // the groups that change corner, one after the other: footprints of two
-        // groups may overlap
         const bool turn = cell != cur;
-        if (__any_sync(0xffffffffu, turn)) {
+        if (ATOMIC) {
+            if (turn) {
+                if (live) warp_flush_atomic<W>(cells, (int)((cur >> 16) * ST + (cur & 0xFFFFu)) + fbase, ar, ai);
+#pragma unroll
+                for (int jx = 0; jx < W; ++jx) ar[jx] = ai[jx] = 0.0f;
+                cur = cell;
+            }
+        } else if (__any_sync(0xffffffffu, turn)) {
+            // the groups that change corner, one after the other: footprints of two
+            // groups may overlap
             unsigned m = __ballot_sync(0xffffffffu, turn && live && j == 0);
             while (m) {
                 if (live && grp * G == __ffs(m) - 1)
@@ -732,8 +757,10 @@ __device__ __forceinline__ void warp_stream(const TileArgs &ta, uint32_t r0, uin
         cell = ncell;
     }
 #pragma unroll 1
-    for (int h = 0; h < NGR; ++h) {
-        if (live && grp == h)
+    for (int h = 0; h < (ATOMIC ? 1 : NGR); ++h) {
+        if (ATOMIC && live)
+            warp_flush_atomic<W>(cells, (int)((cur >> 16) * ST + (cur & 0xFFFFu)) + fbase, ar, ai);
+        if (!ATOMIC && live && grp == h)
             warp_flush<W>(cells, (int)((cur >> 16) * ST + (cur & 0xFFFFu)) + fbase, ar, ai);
         __syncwarp();
     }
@@ -1197,7 +1224,7 @@ static TileArgs make_tile_args(const rick_plan *plan, const WsPtrs &w, const uin
 
 static void set_sub_args(GridArgs &a, const rick_params &p, const WsPtrs &w)
 {
-    a.sub = rick_sub_shape(p.tile);
+    a.sub = rick_sub_shape(&p);
     a.suboff = w.suboff;
     a.items = w.items;
     a.groups = w.groups;
