@@ -550,7 +550,7 @@ def run_ours(args, wl):
     sm_mhz = (m["clocks"] or {}).get("sm_mhz") or (m["clocks"] or {}).get("sm_max_mhz") or 2070.0
     roofs = stage_rooflines(wl, m, rates, sms, sm_mhz, peak)
     dom = max(stage_ms, key=lambda k: stage_ms[k])
-    kernel_name = {"bin": "rick_bin (all binning kernels)", "grid": "grid_kernel",
+    kernel_name = {"bin": "rick_bin (all binning kernels)", "grid": "grid_warps_kernel",
                    "fft_wcorrect": "fft_rows_kernel + fft_cols_kernel"}[dom]
     roofline = {**roofs[dom], "kernel": kernel_name, "stage": dom,
                 "traffic": traffic_of(dom, n_vis), "algorithmic_bytes": alg[dom],

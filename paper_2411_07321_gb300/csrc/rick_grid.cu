@@ -900,7 +900,7 @@ __device__ __forceinline__ uint32_t next_warp(uint32_t *counter)
 // has no FP32 add) and visited the records near a tile's edge once per tile they
 // reach.  16 x 16 corners a subtile leave 32 warps an SM.  On a GB300, against the
 // CTA tiles: 5e7 visibilities of 16 channels, W = 7: 1.92 -> 1.24 ms; 2e8 of 64,
-// W = 9: 9.21 -> 6.81; 1e7 of 4: 0.68 -> 0.35; 4e6 of one: 0.61 -> 0.33; 1e6 of 4:
+// W = 9: 9.21 -> 6.59; 1e7 of 4: 0.68 -> 0.35; 4e6 of one: 0.61 -> 0.33; 1e6 of 4:
 // 106 -> 52 us; 1e4: 58 -> 20 us.  Four CTAs an SM up to W = 10 (W = 9 at three:
 // 2 % slower).
 template <int W>
