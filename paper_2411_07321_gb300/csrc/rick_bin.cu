@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(256) bin_init_kernel(WsPtrs w, uint64_t n_vis,
         hdr->sub_cap = sub_cap;
         hdr->n_items = 0;
         hdr->n_groups = 0;
+        hdr->n_slots = 0;
         hdr->n_vis = n_vis;
         hdr->n_src = n_src;
         hdr->mirror = (uint32_t)mirror;
@@ -909,10 +910,12 @@ __global__ void tile_count_kernel(const uint32_t *off, uint32_t *gcnt, uint32_t 
     dcnt[t] = c.y;
 }
 
-// Append entries (s0 + lane of the owner, first[owner] + step i) for the cnt of
-// every lane to a list, i < cnt: one atomic per warp, all lanes writing.
-__device__ __forceinline__ void append_items(uint32_t cnt, uint32_t from, uint32_t step, uint32_t s0,
-                                             uint32_t *counter, uint2 *list)
+// Room for the cnt entries of every lane in a list of *counter entries, in lane order:
+// the first of each lane's, and of the warp's (total entries).  One atomic per warp.
+struct Entries {
+    uint32_t lane, warp, total;
+};
+__device__ __forceinline__ Entries reserve(uint32_t cnt, uint32_t *counter)
 {
     const int lane = threadIdx.x & 31;
     uint32_t inc = cnt;
@@ -921,31 +924,35 @@ __device__ __forceinline__ void append_items(uint32_t cnt, uint32_t from, uint32
         const uint32_t v = __shfl_up_sync(FULL, inc, o);
         if (lane >= o) inc += v;
     }
-    const uint32_t tot = __shfl_sync(FULL, inc, 31), first = inc - cnt;
-    if (!tot) return;
     uint32_t at = 0;
-    if (lane == 31) at = atomicAdd(counter, tot);
+    if (lane == 31 && inc) at = atomicAdd(counter, inc);
     at = __shfl_sync(FULL, at, 31);
-    for (uint32_t i0 = 0; i0 < tot; i0 += 32) {
+    return {at + inc - cnt, at, __shfl_sync(FULL, inc, 31)};
+}
+
+// put(entry, owning lane, its number among the lane's) for the warp's entries, all lanes
+// at it (put may shuffle; entries past the last are not to be stored).
+template <typename Put>
+__device__ __forceinline__ void each_entry(const Entries &e, Put put)
+{
+    for (uint32_t i0 = 0; i0 < e.total; i0 += 32) {
         // entry i belongs to the last lane whose entries start at or before it
-        const uint32_t i = i0 + lane;
+        const uint32_t i = e.warp + i0 + (threadIdx.x & 31);
         int own = 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
-            own += __shfl_sync(FULL, first, own + o) <= i ? o : 0;
-        const uint32_t k = i - __shfl_sync(FULL, first, own);
-        const uint32_t c = __shfl_sync(FULL, from, own) + step * k;
-        if (i < tot) list[at + i] = make_uint2(s0 + own, c);
+            own += __shfl_sync(FULL, e.lane, own + o) <= i ? o : 0;
+        put(i, own, i - __shfl_sync(FULL, e.lane, own));
     }
 }
 
 // The plain gridding kernel's work items, in no particular order: a thread per
 // subtile counts its records (its class-0 sub-bin and, in the last column and
-// row of subtiles, those of the other classes).
-// All lanes of a warp, s consecutive.
-__device__ __forceinline__ void sub_items(uint32_t s, const uint32_t *suboff, uint32_t nsubtiles,
-                                          const SubShape &sub, uint32_t cap, uint32_t *n_items,
-                                          uint2 *items, uint32_t *n_groups, uint2 *groups)
+// row of subtiles, those of the other classes).  len: the lengths of the lists of
+// groups, single items and slots.  All lanes of a warp, s consecutive.
+__device__ __forceinline__ void sub_items(uint32_t s, uint32_t nsubtiles, const SubShape &sub,
+                                          uint32_t cap, uint32_t nslots, uint32_t *const (&len)[3],
+                                          const WsPtrs &w)
 {
     uint32_t cnt = 0;
     if (s < nsubtiles) {
@@ -953,21 +960,34 @@ __device__ __forceinline__ void sub_items(uint32_t s, const uint32_t *suboff, ui
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             const int64_t id = rick_subtile_range(sub, s, g);
-            if (id >= 0) n += suboff[id + 1] - suboff[id];
+            if (id >= 0) n += w.suboff[id + 1] - w.suboff[id];
         }
         cnt = rick_sub_chunks(n, cap);
     }
-    const uint32_t s0 = s - (threadIdx.x & 31), ng = cnt / RICK_SUB_GROUP;
-    append_items(ng, 0, RICK_SUB_GROUP, s0, n_groups, groups);
-    append_items(cnt - ng * RICK_SUB_GROUP, ng * RICK_SUB_GROUP, 1, s0, n_items, items);
+    const uint32_t s0 = s - (threadIdx.x & 31), ng = cnt / RICK_SUB_GROUP, ns = rick_sub_slots(ng);
+    uint32_t slot = ~0u;
+    if (__any_sync(FULL, ns != 0)) {
+        const uint32_t at = reserve(ns, len[2]).lane;
+        if (ns && at + ns <= nslots) slot = at;
+    }
+    const Entries eg = reserve(ng, len[0]);
+    each_entry(eg, [&](uint32_t i, int own, uint32_t k) {
+        const uint32_t first = __shfl_sync(FULL, slot, own), all = __shfl_sync(FULL, ng, own);
+        if (i < eg.warp + eg.total)
+            w.groups[i] = make_uint4(s0 + own, RICK_SUB_GROUP * k, first, all);
+    });
+    const Entries es = reserve(cnt - ng * RICK_SUB_GROUP, len[1]);
+    each_entry(es, [&](uint32_t i, int own, uint32_t k) {
+        const uint32_t c = __shfl_sync(FULL, ng, own) * RICK_SUB_GROUP + k;
+        if (i < es.warp + es.total) w.items[i] = make_uint2(s0 + own, c);
+    });
 }
 
-__global__ void __launch_bounds__(256) sub_items_kernel(const uint32_t *suboff, uint32_t nsubtiles,
-                                                        SubShape sub, WsHeader *hdr, uint2 *items,
-                                                        uint2 *groups)
+__global__ void __launch_bounds__(256) sub_items_kernel(WsPtrs w, uint32_t nsubtiles, SubShape sub,
+                                                        uint32_t nslots)
 {
-    sub_items(blockIdx.x * blockDim.x + threadIdx.x, suboff, nsubtiles, sub, hdr->sub_cap,
-              &hdr->n_items, items, &hdr->n_groups, groups);
+    uint32_t *const len[3] = {&w.hdr->n_groups, &w.hdr->n_items, &w.hdr->n_slots};
+    sub_items(blockIdx.x * blockDim.x + threadIdx.x, nsubtiles, sub, w.hdr->sub_cap, nslots, len, w);
 }
 
 // Exclusive scan of n values by one CTA of 1024 threads, eight consecutive values a
@@ -1021,7 +1041,7 @@ struct SmallArgs {
     WsPtrs w;
     SubShape sub;
     int nparts, unit_weights, nt, plain;
-    uint32_t ntiles, cap;
+    uint32_t ntiles, cap, nslots;
     int64_t nsubs, nbins;
     rick_bin_stats *stats_out;
 };
@@ -1044,16 +1064,18 @@ __global__ void __launch_bounds__(1024) bin_small_kernel(SmallArgs a)
              [&](int64_t t, uint32_t v) { w.dbase[t] = v; });
     if (a.plain) {
         // the lists' lengths in shared memory until they are known
-        __shared__ uint32_t s_len[2];
-        if (threadIdx.x < 2) s_len[threadIdx.x] = 0;
+        __shared__ uint32_t s_len[3];
+        if (threadIdx.x < 3) s_len[threadIdx.x] = 0;
         __syncthreads();
         const uint32_t ns = a.ntiles << (2 * a.sub.lq), cap = w.hdr->sub_cap;
+        uint32_t *const len[3] = {&s_len[0], &s_len[1], &s_len[2]};
         for (uint32_t s = threadIdx.x; s < ((ns + 31) & ~31u); s += 1024)
-            sub_items(s, w.suboff, ns, a.sub, cap, &s_len[0], w.items, &s_len[1], w.groups);
+            sub_items(s, ns, a.sub, cap, a.nslots, len, w);
         __syncthreads();
         if (threadIdx.x == 0) {
-            w.hdr->n_items = s_len[0];
-            w.hdr->n_groups = s_len[1];
+            w.hdr->n_groups = s_len[0];
+            w.hdr->n_items = s_len[1];
+            w.hdr->n_slots = s_len[2];
         }
     }
 }
@@ -1083,7 +1105,8 @@ static rick_status launch_offsets(rick_plan *plan, const WsPtrs &w, const WsLayo
 {
     if (small) {
         const SmallArgs a = {w, sub, nparts, unit_weights, plan->p.n / plan->p.tile,
-                             rick_grid_plain(&plan->p), (uint32_t)L.ntiles, cap, L.nsubs, L.nbins,
+                             rick_grid_plain(&plan->p), (uint32_t)L.ntiles, cap,
+                             (uint32_t)L.nslots, L.nsubs, L.nbins,
                              stats_out};
         bin_small_kernel<<<1, 1024, 0, st>>>(a);
         RICK_LAUNCH_CHECK(plan);
@@ -1110,7 +1133,7 @@ static rick_status launch_lists(rick_plan *plan, const WsPtrs &w, const WsLayout
     if (!rick_grid_plain(&plan->p)) return RICK_OK;
     const SubShape sub = rick_sub_shape(&plan->p);
     const uint32_t ns = (uint32_t)(L.ntiles << (2 * sub.lq));
-    sub_items_kernel<<<(ns + 255) / 256, 256, 0, st>>>(w.suboff, ns, sub, w.hdr, w.items, w.groups);
+    sub_items_kernel<<<(ns + 255) / 256, 256, 0, st>>>(w, ns, sub, (uint32_t)L.nslots);
     RICK_LAUNCH_CHECK(plan);
     return RICK_OK;
 }

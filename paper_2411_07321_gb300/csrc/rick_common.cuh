@@ -125,13 +125,13 @@ struct WsHeader {
     uint32_t mc_count;                  // tiles gridded by several work items
     // plain gridding: records per chunk; work items and the work counters,
     // of a warp and of a CTA
-    uint32_t sub_cap, n_items, item_next, n_groups, group_next;
+    uint32_t sub_cap, n_items, item_next, n_groups, group_next, n_slots;
 };
 
 struct WsLayout {
     size_t header, key, rank, cell, frac, perm, rec, rcell, hist, suboff, offsets, gbase, dbase, scan,
-        wpart, bkey, wplane, dkey, didx, dkey2, dcnt, vpart, mcslot, mcacc, items, groups, total;
-    int64_t n_vis, nbins, nsubs, nitems, ngroups, ntiles, nscan, nkeyblocks, ndetblocks;
+        wpart, bkey, wplane, dkey, didx, dkey2, dcnt, vpart, mcslot, mcacc, items, groups, slots, arrived, total;
+    int64_t n_vis, nbins, nsubs, nitems, ngroups, nslots, ntiles, nscan, nkeyblocks, ndetblocks;
 };
 
 // Key pass blocks: 1024 visibilities, staged in 28 KB of shared memory, so that
@@ -205,21 +205,35 @@ RICK_HD int64_t rick_subtile_range(const SubShape &s, uint32_t id, int g)
 }
 
 // Work of the plain gridding kernel: a subtile's records in chunks of at most
-// sub_cap, cut evenly.  Eight chunks of a subtile make a CTA's item -- a warp
+// sub_cap, cut evenly.  Eight chunks of a subtile make a CTA's item (a group) -- a warp
 // each, summed across the warps before they go to the planes -- and what is left
-// a warp's items.  (Every chunk by itself puts hundreds of partial sums, one
-// after the other, onto the cells of the array core: the image of 2e8
-// visibilities on 8192^2 was then 4.5 times further from its 64-bit value.)
-// About four chunks per resident warp.  At most 2048 records, where the partial
-// sums are few enough (2e8 visibilities, 512 / 1024 / 2048 records: error of the
-// image 2.5e-5 / 1.3e-5 / 1.1e-5; 1.3e-5 with CTA tiles of 20559 records).  At
+// a warp's items.  About four chunks per resident warp; at most 2048 records.  At
 // least 128, where items begin to cost more in list and reductions than they
-// balance (1e6 visibilities, 128 / 64: 50 / 55 us), or 64 for the small sets, where
-// an item's steps are the call's latency (1e4 visibilities, 64 / 128 / 512: 21 /
-// 31 / 96 us).
+// balance (1e6 visibilities, 128 / 64: 50 / 55 us); less where that leaves warps without
+// any (an item's steps are then the call's latency), down to 32.
+//
+// Each FP32 add of a partial sum to a plane rounds the whole sum so far, and the core of
+// an array has tens to hundreds of groups on a subtile: the error of the image of 1e6
+// visibilities was that of a few cells, and differed twofold from call to call with the
+// order of their adds.  A subtile of RICK_SLOT_GROUPS groups and more therefore has slots
+// of its own, one for each eight groups up to 16 (rick_sub_slots); the last of its groups
+// adds the slots up in FP64 and takes the sum to the planes.  Error of the image against
+// 64 bits, mean / largest of 32 calls on the worst of four sets, 1e6 visibilities on
+// 1024^2: 3.4e-7 / 3.7e-7 (without slots 6.8 / 8.5; tile by tile 7.1 / 9.5); 65536 on
+// 256^2: 4.5e-7 / 5.3e-7 (8.0 / 13.2; 7.0 / 11.4).  It costs the gridding 2 us on the
+// smaller, 4 on the larger and 1 to 4 % above.  At most RICK_SLOTS_MAX slots (16 MB),
+// first come; the other groups add to the planes.
 #define RICK_SUB_GROUP 8
-#define RICK_SUB_CAP_MIN 64
+#define RICK_SUB_CAP_MIN 32
 #define RICK_SUB_CAP_MAX 2048
+#define RICK_SLOT_GROUPS 8
+#define RICK_SLOTS_MAX 2048
+#define RICK_SLOT_STRIDE 32  // cells of a slot's row (31 at the widest support); even
+#define RICK_SLOT_CELLS (31 * RICK_SLOT_STRIDE)
+RICK_HD uint32_t rick_sub_slots(uint32_t groups)
+{
+    return groups < RICK_SLOT_GROUPS ? 0 : groups < 8 * 16 ? (groups + 7) / 8 : 16;
+}
 RICK_HD uint32_t rick_sub_chunks(uint32_t n, uint32_t cap) { return (n + cap - 1) / cap; }
 static inline uint32_t rick_sub_cap(int64_t n_vis, int num_sms)
 {
@@ -286,12 +300,17 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
     L.ndetblocks = det ? (n_vis + RICK_DET_BLOCK - 1) / RICK_DET_BLOCK : 0;
     const SubShape sub = rick_sub_shape(p);
     L.nsubs = L.ntiles * sub.per;
-    // work items: at most one per subtile that holds records, and one more per
-    // RICK_SUB_CAP_MIN records
-    L.nitems = L.ntiles << (2 * sub.lq);
-    if (L.nitems > n_vis) L.nitems = n_vis;
-    L.nitems += n_vis / RICK_SUB_CAP_MIN + 1;
-    L.ngroups = n_vis / (RICK_SUB_GROUP - 1) / RICK_SUB_CAP_MIN + 1;
+    L.nitems = L.ngroups = L.nslots = 0;
+    if (rick_grid_plain(p)) {
+        // work items: at most one per subtile that holds records, and one more per
+        // RICK_SUB_CAP_MIN records
+        L.nitems = L.ntiles << (2 * sub.lq);
+        if (L.nitems > n_vis) L.nitems = n_vis;
+        L.nitems += n_vis / RICK_SUB_CAP_MIN + 1;
+        L.ngroups = n_vis / (RICK_SUB_GROUP - 1) / RICK_SUB_CAP_MIN + 1;
+        L.nslots = 2 * L.ngroups / RICK_SLOT_GROUPS;
+        if (L.nslots > RICK_SLOTS_MAX) L.nslots = RICK_SLOTS_MAX;
+    }
     L.nscan = rick_scan_tmp(L.nsubs + 1);
     if (det) {
         const int64_t d = rick_scan_tmp((1 << RICK_DET_DIGIT) * L.ndetblocks + 1);
@@ -329,7 +348,9 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
     L.mcslot = o; o += rick_align256(det ? 4 * (size_t)(L.ntiles + 1) : 0);
     L.mcacc = o;  o += rick_align256(16 * (size_t)rick_det_slots(p, n_vis) * p->tile * p->tile);
     L.items = o;  o += rick_align256(8 * (size_t)L.nitems);
-    L.groups = o; o += rick_align256(8 * (size_t)L.ngroups);
+    L.groups = o; o += rick_align256(16 * (size_t)L.ngroups);
+    L.slots = o;  o += rick_align256(8 * (size_t)L.nslots * RICK_SLOT_CELLS);
+    L.arrived = o; o += rick_align256(4 * (size_t)L.nslots);
     L.total = o;
     return L;
 }
@@ -346,7 +367,10 @@ struct WsPtrs {
     uint32_t *dkey, *didx, *dkey2, *dcnt, *mcslot;  // deterministic mode
     double *vpart;
     unsigned long long *mcacc;
-    uint2 *items, *groups;  // plain gridding: (subtile, first chunk) of each work item
+    uint2 *items;       // plain gridding: (subtile, chunk) of each single item
+    uint4 *groups;      // (subtile, first chunk, its first slot or ~0, its groups)
+    float2 *slots;      // RICK_SLOT_CELLS each
+    uint32_t *arrived;  // groups that have added to the slots (at the first one)
 };
 
 static inline WsPtrs rick_ws_ptrs(void *ws, const WsLayout &L)
@@ -378,7 +402,9 @@ static inline WsPtrs rick_ws_ptrs(void *ws, const WsLayout &L)
     w.mcslot = (uint32_t *)(b + L.mcslot);
     w.mcacc = (unsigned long long *)(b + L.mcacc);
     w.items = (uint2 *)(b + L.items);
-    w.groups = (uint2 *)(b + L.groups);
+    w.groups = (uint4 *)(b + L.groups);
+    w.slots = (float2 *)(b + L.slots);
+    w.arrived = (uint32_t *)(b + L.arrived);
     return w;
 }
 

@@ -34,7 +34,11 @@ struct GridArgs {
     uint32_t nzero;  // tile-clearing items (RICK_ZERO_GROUP tiles each); 0 when accumulating
     SubShape sub;            // plain sums: subtiles, their record offsets, the work items
     const uint32_t *suboff;
-    const uint2 *items, *groups;
+    const uint2 *items;
+    const uint4 *groups;
+    float2 *slots;  // sums of dense subtiles
+    uint32_t *arrived;
+    uint32_t nslots;
     const uint32_t *mcslot;     // deterministic mode: slot of each multi-item tile
     unsigned long long *mcacc;  // deterministic mode: the slots' int64 (re, im) sums
 };
@@ -813,18 +817,36 @@ __device__ __forceinline__ void grid_chunk(const GridArgs &a, uint32_t id, uint3
     }
 }
 
+// Two cells of a subtile's row, col even, added to its cells in the planes or a slot (row
+// stride n) -- the checkerboard (-1)^(i+j) folded in (the subtile's first row and column
+// are even); nothing where both are zero, as cells are that no footprint reached, those
+// off the grid among them.
+__device__ __forceinline__ void add_cells(float2 *out, int n, int row, int col, float2 u, float2 v)
+{
+    if (u.x != 0.0f || u.y != 0.0f || v.x != 0.0f || v.y != 0.0f) {
+        if (row & 1) {
+            u.x = -u.x;
+            u.y = -u.y;
+        } else {
+            v.x = -v.x;
+            v.y = -v.y;
+        }
+        atomicAdd((float4 *)(out + (size_t)row * n + col), make_float4(u.x, u.y, v.x, v.y));
+    }
+}
+
+__device__ __forceinline__ float2 *sub_cells(const GridArgs &a, uint32_t id)
+{
+    const SubOrigin so = sub_origin(a, id);
+    return a.planes + ((size_t)so.k * a.t.n + so.y0) * a.t.n + so.x0;
+}
+
 // The sums of nc sets of a subtile's cells (strides of SubCells::CELLS) added to
-// the planes and the cells zeroed, by threads t of nt: two cells of a row at a
-// time, the checkerboard (-1)^(i+j) folded in (x0, y0 and the column are even);
-// cells that no footprint reached are zero, those off the grid among them.
+// out and the cells zeroed, by threads t of nt: two cells of a row at a time.
 template <int W>
-__device__ __forceinline__ void cells_out(const GridArgs &a, uint32_t id, float2 *cells, int nc,
-                                          int t, int nt)
+__device__ __forceinline__ void cells_out(float2 *out, int n, float2 *cells, int nc, int t, int nt)
 {
     constexpr int ROWS = SubCells<W>::ROWS, ST = SubCells<W>::STRIDE, HP = (ROWS + 1) / 2;
-    const SubOrigin so = sub_origin(a, id);
-    const int n = a.t.n;
-    float2 *plane = a.planes + ((size_t)so.k * n + so.y0) * n + so.x0;
     for (int i = t; i < ROWS * HP; i += nt) {
         const int row = i / HP, col = 2 * (i - row * HP);
         const bool two = ROWS % 2 == 0 || col + 1 < ROWS;
@@ -839,49 +861,71 @@ __device__ __forceinline__ void cells_out(const GridArgs &a, uint32_t id, float2
                 p[1] = make_float2(0.0f, 0.0f);
             }
         }
-        if (u.x != 0.0f || u.y != 0.0f || v.x != 0.0f || v.y != 0.0f) {
-            if (row & 1) {
-                u.x = -u.x;
-                u.y = -u.y;
-            } else {
-                v.x = -v.x;
-                v.y = -v.y;
-            }
-            atomicAdd((float4 *)(plane + (size_t)row * n + col), make_float4(u.x, u.y, v.x, v.y));
-        }
+        add_cells(out, n, row, col, u, v);
     }
 }
 
-// A work item: of the CTA (a chunk per warp, one sum; all threads call it) or, with
-// single, of the warp.  cells: the CTA's.
+// The CTA's group: the subtile, its slot (~0: the planes), the subtile's first slot and
+// number of groups, its job of a batch; and whether it was the last of its subtile's to
+// arrive.
+struct GroupItem {
+    uint32_t index, id, slot, first, all;
+    int job;
+    bool last;
+    uint32_t total[2];  // groups and single items of all jobs
+};
+
+// The slots of a subtile whose groups have all arrived added up and to the planes.
 template <int W>
-__device__ __forceinline__ void grid_item(const GridArgs &a, bool single, uint2 item, float2 *cells,
-                                          const float2 *coef2)
+__device__ __forceinline__ void slots_out(const GridArgs &a, const volatile GroupItem &g)
 {
-    // (the subtile waits in shared memory: the record loop needs the registers)
-    __shared__ volatile uint32_t s_id[RICK_GRID_WARPS];
-    const int wid = threadIdx.x >> 5;
-    float2 *own = cells + wid * SubCells<W>::CELLS;
-    s_id[wid] = item.x;
-    grid_chunk<W>(a, item.x, item.y + (single ? 0 : wid), own, coef2);
-    if (single)
-        __syncwarp();
-    else
-        __syncthreads();
-    cells_out<W>(a, s_id[wid], single ? own : cells, single ? 1 : RICK_GRID_WARPS,
-                 single ? threadIdx.x & 31 : threadIdx.x, single ? 32 : 32 * RICK_GRID_WARPS);
-    __syncwarp();
+    constexpr int ROWS = SubCells<W>::ROWS, HP = (ROWS + 1) / 2;
+    const uint32_t ns = rick_sub_slots(g.all);
+    const float2 *first = a.slots + (size_t)g.first * RICK_SLOT_CELLS;
+    float2 *out = sub_cells(a, g.id);
+    for (int i = threadIdx.x; i < ROWS * HP; i += 32 * RICK_GRID_WARPS) {
+        const int row = i / HP, col = 2 * (i - row * HP);
+        const float4 *p = (const float4 *)(first + row * RICK_SLOT_STRIDE + col);
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (uint32_t k = 0; k < ns; ++k) {
+            const float4 v = __ldcg(p + k * (RICK_SLOT_CELLS / 2));
+            s[0] += v.x;
+            s[1] += v.y;
+            s[2] += v.z;
+            s[3] += v.w;
+        }
+        // (signed for the checkerboard already; no footprint reaches a zero cell)
+        if (s[0] != 0.0 || s[1] != 0.0 || s[2] != 0.0 || s[3] != 0.0)
+            atomicAdd((float4 *)(out + (size_t)row * a.t.n + col),
+                      make_float4((float)s[0], (float)s[1], (float)s[2], (float)s[3]));
+    }
 }
 
-// Take the next item of a counter: for the whole CTA, or for each warp.
-__device__ __forceinline__ uint32_t next_cta(uint32_t *counter)
+// The next group, for the whole CTA; total[0] or more after the last.  Counts the one
+// before in at its subtile's slots, and sends them to the planes if it was the last.
+template <int W, typename Jobs>
+__device__ __forceinline__ uint32_t next_group(const Jobs &jobs, volatile GroupItem &g)
 {
-    __shared__ uint32_t s_next;
-    __syncthreads();  // the cells are zero again, the last index has been read
-    if (threadIdx.x == 0) s_next = atomicAdd(counter, 1u);
+    __syncthreads();  // the cells are zero again, the last item has been read
+    if (threadIdx.x == 0) {
+        g.index = atomicAdd(&jobs.hdr()->group_next, 1u);
+        g.last = false;
+        if (g.slot != ~0u) {
+            __threadfence();  // the CTA's sums before its count
+            g.last = atomicAdd(&jobs.args(g.job).arrived[g.first], 1u) == g.all - 1;
+        }
+    }
     __syncthreads();
-    return s_next;
+    if (g.last) {
+        __threadfence();
+        slots_out<W>(jobs.args(g.job), g);
+        __syncthreads();
+    }
+    return g.index;
 }
+
+// The next single item, for each warp.
 __device__ __forceinline__ uint32_t next_warp(uint32_t *counter)
 {
     uint32_t b = 0;
@@ -889,9 +933,87 @@ __device__ __forceinline__ uint32_t next_warp(uint32_t *counter)
     return __shfl_sync(0xffffffffu, b, 0);
 }
 
-// Plain sums: the CTAs take the groups of chunks from a counter in the workspace
-// header (reset by zero_tiles_kernel, launched just before), then each warp takes
-// single chunks from another until none is left.
+// The plain kernels' work: the CTAs take the groups of chunks from a counter in the
+// workspace header (reset by zero_tiles_kernel, launched just before), then each warp
+// takes single chunks from another until none is left.
+template <int W, typename Jobs>
+__device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
+{
+    // (what the sums go to waits in shared memory: the record loop needs the registers)
+    __shared__ volatile uint32_t s_id[RICK_GRID_WARPS], s_slot[RICK_GRID_WARPS];
+    __shared__ volatile GroupItem s_group;
+    const int wid = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < RICK_GRID_WARPS * SubCells<W>::CELLS; i += 32 * RICK_GRID_WARPS)
+        cells[i] = make_float2(0.0f, 0.0f);
+    if (threadIdx.x == 0) s_group.slot = ~0u;
+    if (threadIdx.x < 2) s_group.total[threadIdx.x] = jobs.total(threadIdx.x);
+    float2 coef2[RICK_POLY_N];
+    load_coef<W>(jobs.args(0).t.kp, coef2);
+    int cur = 0;
+    bool single = false;
+#pragma unroll 1
+    for (;;) {
+        uint32_t b = 0, id, chunk, slot = ~0u;
+        if (!single) {
+            b = next_group<W>(jobs, s_group);
+            single = b >= s_group.total[0];
+        }
+        if (single) {
+            b = next_warp(&jobs.hdr()->item_next);
+            if (b >= s_group.total[1]) break;
+        }
+        const int j = jobs.job(b, single);
+        if (single) {
+            const uint2 q = jobs.args(j).items[b - jobs.first(j, true)];
+            id = q.x;
+            chunk = q.y;
+        } else {
+            const uint4 q = jobs.args(j).groups[b - jobs.first(j, false)];
+            id = q.x;
+            chunk = q.y + wid;
+            if (q.z != ~0u) slot = q.z + q.y / RICK_SUB_GROUP % rick_sub_slots(q.w);
+            if (threadIdx.x == 0) {
+                s_group.job = j;
+                s_group.id = id;
+                s_group.slot = slot;
+                s_group.first = q.z;
+                s_group.all = q.w;
+            }
+        }
+        const GridArgs &a = jobs.args(j);
+        if (j != cur) load_coef<W>(a.t.kp, coef2);
+        cur = j;
+        s_id[wid] = id;
+        s_slot[wid] = slot;
+        float2 *own = cells + wid * SubCells<W>::CELLS;
+        grid_chunk<W>(a, id, chunk, own, coef2);
+        if (single)
+            __syncwarp();
+        else
+            __syncthreads();
+        slot = s_slot[wid];
+        cells_out<W>(slot == ~0u ? sub_cells(a, s_id[wid]) : a.slots + (size_t)slot * RICK_SLOT_CELLS,
+                     slot == ~0u ? a.t.n : RICK_SLOT_STRIDE, single ? own : cells,
+                     single ? 1 : RICK_GRID_WARPS, single ? threadIdx.x & 31 : threadIdx.x,
+                     single ? 32 : 32 * RICK_GRID_WARPS);
+        __syncwarp();
+    }
+}
+
+// One job (job 0).
+struct OneJob {
+    const GridArgs &a;
+    __device__ __forceinline__ const GridArgs &args(int) const { return a; }
+    __device__ __forceinline__ WsHeader *hdr() const { return a.t.hdr; }
+    __device__ __forceinline__ uint32_t total(bool single) const
+    {
+        return single ? a.t.hdr->n_items : a.t.hdr->n_groups;
+    }
+    __device__ __forceinline__ int job(uint32_t, bool) const { return 0; }
+    __device__ __forceinline__ uint32_t first(int, bool) const { return 0; }
+};
+
+// Plain sums.
 //
 // Bound by instruction issue (62 % of cycles; long_scoreboard, the record loads,
 // is the first stall).  A warp owns its cells, so a corner change costs W loads
@@ -908,20 +1030,7 @@ __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_warps_kernel(const __grid_constant__ GridArgs a)
 {
     extern __shared__ float2 s_cells[];
-    float2 coef2[RICK_POLY_N];
-    load_coef<W>(a.t.kp, coef2);
-    for (int i = threadIdx.x; i < RICK_GRID_WARPS * SubCells<W>::CELLS; i += 32 * RICK_GRID_WARPS)
-        s_cells[i] = make_float2(0.0f, 0.0f);
-    WsHeader *hdr = a.t.hdr;
-#pragma unroll 1
-    for (int single = 0; single < 2; ++single) {
-        const uint32_t total = single ? hdr->n_items : hdr->n_groups;
-        for (;;) {
-            const uint32_t b = single ? next_warp(&hdr->item_next) : next_cta(&hdr->group_next);
-            if (b >= total) break;
-            grid_item<W>(a, single, single ? a.items[b] : a.groups[b], s_cells, coef2);
-        }
-    }
+    plain_work<W>(OneJob{a}, s_cells);
 }
 
 // Several imaging jobs gridded by one launch (rick_grid_sparse_batch): the jobs'
@@ -946,6 +1055,16 @@ __device__ __forceinline__ void clear_tile(float2 *planes, uint32_t t, int nt, i
         tile[(size_t)(i >> lh) * (n / 2) + (i & ((1 << lh) - 1))] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
+// The slots of the last binning's dense subtiles zeroed, by block b of nb.
+__device__ __forceinline__ void clear_slots(const WsHeader *hdr, float2 *slots, uint32_t *arrived,
+                                            uint32_t nslots, uint32_t b, uint32_t nb)
+{
+    const uint32_t used = min(hdr->n_slots, nslots), first = b * blockDim.x + threadIdx.x;
+    for (uint32_t i = first; i < used * (RICK_SLOT_CELLS / 2); i += nb * blockDim.x)
+        ((float4 *)slots)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (uint32_t i = first; i < used; i += nb * blockDim.x) arrived[i] = 0;
+}
+
 #define RICK_ZERO_LOOK 8
 
 // Zero the tiles of at least `least` work items, into which the grid kernel adds,
@@ -963,7 +1082,9 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
                                                          WsHeader *hdr, int accumulate,
                                                          const uint32_t *mcslot,
                                                          unsigned long long *mcacc,
-                                                         const uint8_t *touched, uint32_t least)
+                                                         const uint8_t *touched, uint32_t least,
+                                                         float2 *slots, uint32_t *arrived,
+                                                         uint32_t nslots)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hdr->grid_next = 0;
@@ -972,6 +1093,7 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
         hdr->group_next = 0;
     }
     const int lane = threadIdx.x & 31, T = 1 << log2T;
+    if (nslots) clear_slots(hdr, slots, arrived, nslots, blockIdx.x, gridDim.x);
     if (!mcacc && accumulate) return;
     // a block looks at RICK_ZERO_LOOK tiles at a time, and its warps share the rows
     // of each one to clear: the tiles with records lie side by side
@@ -1005,6 +1127,7 @@ __global__ void __launch_bounds__(256)
         ta.hdr->group_next = 0;
     }
     const int lane = threadIdx.x & 31;
+    clear_slots(ta.hdr, a.slots, a.arrived, a.nslots, blockIdx.x, gridDim.x);
     for (uint32_t t0 = blockIdx.x * RICK_ZERO_LOOK; t0 < ta.ntiles;
          t0 += gridDim.x * RICK_ZERO_LOOK) {
         const uint32_t tl = t0 + lane;
@@ -1014,10 +1137,25 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// As grid_warps_kernel over the batch's work: entry b of the jobs' lists belongs to
-// the job j with cum[j] <= b < cum[j + 1] (cum: running totals of the jobs'
-// entries), and is that job's entry b - cum[j].  The lanes' kernel coefficients
-// are loaded again when the job changes.
+// The jobs of a batch: entry b of the jobs' lists belongs to the job j with
+// cum[j] <= b < cum[j + 1] (cum: running totals of the jobs' entries), and is that job's
+// entry b - cum[j].
+struct BatchJobs {
+    const GridBatchArgs &ba;
+    const uint32_t (*cum)[RICK_GRID_BATCH_MAX + 1];
+    __device__ __forceinline__ const GridArgs &args(int j) const { return ba.job[j]; }
+    __device__ __forceinline__ WsHeader *hdr() const { return ba.job[0].t.hdr; }
+    __device__ __forceinline__ uint32_t total(bool single) const { return cum[single][ba.n_jobs]; }
+    __device__ __forceinline__ int job(uint32_t b, bool single) const
+    {
+        int j = 0;
+        while (j + 1 < ba.n_jobs && cum[single][j + 1] <= b) ++j;
+        return j;
+    }
+    __device__ __forceinline__ uint32_t first(int j, bool single) const { return cum[single][j]; }
+};
+
+// As grid_warps_kernel over the batch's work.
 template <int W>
 __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_batch_kernel(const __grid_constant__ GridBatchArgs ba)
@@ -1033,27 +1171,8 @@ __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
             s_cum[threadIdx.x][j + 1] = c;
         }
     }
-    for (int i = threadIdx.x; i < RICK_GRID_WARPS * SubCells<W>::CELLS; i += 32 * RICK_GRID_WARPS)
-        s_cells[i] = make_float2(0.0f, 0.0f);
     __syncthreads();
-    float2 coef2[RICK_POLY_N];
-    int cur = -1;
-#pragma unroll 1
-    for (int single = 0; single < 2; ++single) {
-        WsHeader *h0 = ba.job[0].t.hdr;
-        const uint32_t *cum = s_cum[single], total = cum[ba.n_jobs];
-        for (;;) {
-            const uint32_t b = single ? next_warp(&h0->item_next) : next_cta(&h0->group_next);
-            if (b >= total) break;
-            int j = 0;
-            while (j + 1 < ba.n_jobs && cum[j + 1] <= b) ++j;
-            const GridArgs &a = ba.job[j];
-            if (j != cur) load_coef<W>(a.t.kp, coef2);
-            cur = j;
-            grid_item<W>(a, single, single ? a.items[b - cum[j]] : a.groups[b - cum[j]], s_cells,
-                         coef2);
-        }
-    }
+    plain_work<W>(BatchJobs{ba, s_cum}, s_cells);
 }
 
 // Deterministic mode: the tiles gridded by several work items, from their
@@ -1222,12 +1341,15 @@ static TileArgs make_tile_args(const rick_plan *plan, const WsPtrs &w, const uin
     return t;
 }
 
-static void set_sub_args(GridArgs &a, const rick_params &p, const WsPtrs &w)
+static void set_sub_args(GridArgs &a, const rick_params &p, const WsPtrs &w, const WsLayout &L)
 {
     a.sub = rick_sub_shape(&p);
     a.suboff = w.suboff;
     a.items = w.items;
     a.groups = w.groups;
+    a.slots = w.slots;
+    a.arrived = w.arrived;
+    a.nslots = (uint32_t)L.nslots;
 }
 
 static int ilog2(int x)
@@ -1320,7 +1442,8 @@ rick_status rick_grid_impl(rick_plan *plan, void *ws_dev, void *planes_dev, int 
     if (plan->sticky != RICK_OK) return plan->sticky;
     if (((uintptr_t)ws_dev & 255) || ((uintptr_t)planes_dev & 15)) return RICK_EINVAL;
     const rick_params &p = plan->p;
-    WsPtrs w = rick_ws_ptrs(ws_dev, rick_ws_layout(&p, plan->max_vis));
+    const WsLayout L = rick_ws_layout(&p, plan->max_vis);
+    WsPtrs w = rick_ws_ptrs(ws_dev, L);
     cudaStream_t st = (cudaStream_t)stream;
     GridArgs a;
     a.t = make_tile_args(plan, w, w.gbase);
@@ -1335,11 +1458,11 @@ rick_status rick_grid_impl(rick_plan *plan, void *ws_dev, void *planes_dev, int 
     if (det && mode == RICK_GRID_CHUNK_TILES) return RICK_EINVAL;  // its slots add per tile
     a.mcslot = det ? w.mcslot : NULL;
     a.mcacc = det ? w.mcacc : NULL;
-    set_sub_args(a, p, w);
+    set_sub_args(a, p, w, L);
     const uint32_t least = !rick_grid_plain(&p) ? 2u : mode == RICK_GRID_OVERWRITE ? 0u : 1u;
-    zero_tiles_kernel<<<(accumulate && !det) ? 1 : plan->num_sms * 8, 256, 0, st>>>(
+    zero_tiles_kernel<<<(accumulate && !det && !a.nslots) ? 1 : plan->num_sms * 8, 256, 0, st>>>(
         w.gbase, a.t.ntiles, a.t.nt, a.log2T, p.n, a.planes, w.hdr, accumulate, a.mcslot,
-        a.mcacc, a.touched, least);
+        a.mcacc, a.touched, least, a.slots, a.arrived, a.nslots);
     RICK_LAUNCH_CHECK(plan);
     const int gmode = det ? GM_DET : p.precision == RICK_PREC_FP32_COMPENSATED ? GM_COMP : GM_PLAIN;
 #define CALL_GRID(WW) err = launch_grid<WW>(a, gmode, plan->num_sms, st)
@@ -1409,7 +1532,8 @@ extern "C" rick_status rick_grid_sparse_batch(rick_plan *const *plans, void *con
     int tiles_max = 0;
     for (int j = 0; j < n_jobs; ++j) {
         const rick_params &p = plans[j]->p;
-        WsPtrs w = rick_ws_ptrs(ws_dev[j], rick_ws_layout(&p, plans[j]->max_vis));
+        const WsLayout L = rick_ws_layout(&p, plans[j]->max_vis);
+        WsPtrs w = rick_ws_ptrs(ws_dev[j], L);
         GridArgs &a = ba.job[j];
         a.t = make_tile_args(plans[j], w, w.gbase);
         a.planes = (float2 *)planes_dev[j];
@@ -1417,7 +1541,7 @@ extern "C" rick_status rick_grid_sparse_batch(rick_plan *const *plans, void *con
         a.accumulate = 0;
         a.touched = NULL;
         a.nzero = 0;
-        set_sub_args(a, p, w);
+        set_sub_args(a, p, w, L);
         a.mcslot = NULL;
         a.mcacc = NULL;
         tiles_max = max(tiles_max, (int)a.t.ntiles);
