@@ -104,6 +104,9 @@ struct rick_plan {
 // ------------------------------------------------------------------------
 // Workspace layout (caller-owned device buffer, 256-byte aligned pieces)
 
+// Counters of the plain gridding kernel's single items.
+#define RICK_ITEM_COUNTERS 16
+
 struct WsHeader {
     rick_bin_stats stats;               // the stats of the last rick_bin
     unsigned long long wmin_key, wmax_key;  // monotone keys of the w range
@@ -125,7 +128,8 @@ struct WsHeader {
     uint32_t mc_count;                  // tiles gridded by several work items
     // plain gridding: records per chunk; work items and the work counters,
     // of a warp and of a CTA
-    uint32_t sub_cap, n_items, item_next, n_groups, group_next, n_slots;
+    uint32_t sub_cap, n_items, n_groups, group_next, n_slots;
+    uint32_t item_next[RICK_ITEM_COUNTERS][8];  // a sector each
 };
 
 struct WsLayout {

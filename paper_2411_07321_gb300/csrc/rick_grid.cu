@@ -847,6 +847,10 @@ template <int W>
 __device__ __forceinline__ void cells_out(float2 *out, int n, float2 *cells, int nc, int t, int nt)
 {
     constexpr int ROWS = SubCells<W>::ROWS, ST = SubCells<W>::STRIDE, HP = (ROWS + 1) / 2;
+    // (By two, items of a few records take a fifth less -- 1e6 visibilities spread over
+    // 1e5 subtiles, W = 4 / 9: 247 -> 201, 432 -> 396 us -- but at W = 7 the record loop
+    // comes out 3 to 5 % slower: 4e6 visibilities of one channel, 339 -> 356.)
+#pragma unroll(W == 7 ? 1 : 2)
     for (int i = t; i < ROWS * HP; i += nt) {
         const int row = i / HP, col = 2 * (i - row * HP);
         const bool two = ROWS % 2 == 0 || col + 1 < ROWS;
@@ -865,19 +869,39 @@ __device__ __forceinline__ void cells_out(float2 *out, int n, float2 *cells, int
     }
 }
 
-// The CTA's group: the subtile, its slot (~0: the planes), the subtile's first slot and
-// number of groups, its job of a batch; and whether it was the last of its subtile's to
-// arrive.
-struct GroupItem {
+// The work of the plain kernels: groups, a CTA each, then single items, a warp each,
+// `take` at a time.  A CTA begins with the group of its own number, and the warps of a
+// CTA beyond the groups with single items of their own; only what is left is handed out
+// by counters, whose atomics pass one by one (3.5 ns each: with one counter that every
+// warp asks, 1e5 items of a few records took 380 us, and the last requests of 4864 warps
+// 17 us).  A warp asks one of RICK_ITEM_COUNTERS, each for every RICK_ITEM_COUNTERS-th
+// `take` items.
+//
+// And the CTA's group: the subtile, its slot (~0: the planes), the subtile's first slot
+// and number of groups, its job of a batch; and whether it was the last of its subtile's
+// to arrive.
+struct PlainWork {
+    uint32_t total[2];  // groups and single items of all jobs
+    uint32_t take, idle;  // idle: CTAs without a group
     uint32_t index, id, slot, first, all;
     int job;
     bool last;
-    uint32_t total[2];  // groups and single items of all jobs
 };
+
+__device__ __forceinline__ void start_work(volatile PlainWork &w, uint32_t groups, uint32_t singles)
+{
+    const uint32_t share = singles / (gridDim.x * RICK_GRID_WARPS);
+    w.total[0] = groups;
+    w.total[1] = singles;
+    w.take = share >= 64 ? 8u : share >= 16 ? 4u : 1u;
+    w.idle = groups < gridDim.x ? gridDim.x - groups : 0u;
+    w.index = ~0u;
+    w.slot = ~0u;
+}
 
 // The slots of a subtile whose groups have all arrived added up and to the planes.
 template <int W>
-__device__ __forceinline__ void slots_out(const GridArgs &a, const volatile GroupItem &g)
+__device__ __forceinline__ void slots_out(const GridArgs &a, const volatile PlainWork &g)
 {
     constexpr int ROWS = SubCells<W>::ROWS, HP = (ROWS + 1) / 2;
     const uint32_t ns = rick_sub_slots(g.all);
@@ -905,11 +929,12 @@ __device__ __forceinline__ void slots_out(const GridArgs &a, const volatile Grou
 // The next group, for the whole CTA; total[0] or more after the last.  Counts the one
 // before in at its subtile's slots, and sends them to the planes if it was the last.
 template <int W, typename Jobs>
-__device__ __forceinline__ uint32_t next_group(const Jobs &jobs, volatile GroupItem &g)
+__device__ __forceinline__ uint32_t next_group(const Jobs &jobs, volatile PlainWork &g)
 {
     __syncthreads();  // the cells are zero again, the last item has been read
     if (threadIdx.x == 0) {
-        g.index = atomicAdd(&jobs.hdr()->group_next, 1u);
+        g.index = g.index == ~0u ? blockIdx.x
+                : g.idle == 0 ? gridDim.x + atomicAdd(&jobs.hdr()->group_next, 1u) : ~0u - 1;
         g.last = false;
         if (g.slot != ~0u) {
             __threadfence();  // the CTA's sums before its count
@@ -925,28 +950,39 @@ __device__ __forceinline__ uint32_t next_group(const Jobs &jobs, volatile GroupI
     return g.index;
 }
 
-// The next single item, for each warp.
-__device__ __forceinline__ uint32_t next_warp(uint32_t *counter)
+// The warp's next single item after its last one (~0: none yet); ~0 after the last.
+__device__ __forceinline__ uint32_t next_single(WsHeader *hdr, const volatile PlainWork &w,
+                                                uint32_t last)
 {
-    uint32_t b = 0;
-    if ((threadIdx.x & 31) == 0) b = atomicAdd(counter, 1u);
-    return __shfl_sync(0xffffffffu, b, 0);
+    const uint32_t total = w.total[1], take = w.take, idle = w.idle, wid = threadIdx.x >> 5;
+    uint32_t b = last + 1;
+    if (last == ~0u && gridDim.x - blockIdx.x <= idle) {
+        b = (wid * idle + gridDim.x - 1 - blockIdx.x) * take;
+    } else if (last == ~0u || b % take == 0) {
+        const uint32_t first = RICK_GRID_WARPS * idle;
+        if (first * take >= total) return ~0u;
+        const uint32_t k = (blockIdx.x * RICK_GRID_WARPS + wid) % RICK_ITEM_COUNTERS;
+        if ((threadIdx.x & 31) == 0)
+            b = (first + k + RICK_ITEM_COUNTERS * atomicAdd(&hdr->item_next[k][0], 1u)) * take;
+        b = __shfl_sync(0xffffffffu, b, 0);
+    }
+    return b < total ? b : ~0u;
 }
 
-// The plain kernels' work: the CTAs take the groups of chunks from a counter in the
-// workspace header (reset by zero_tiles_kernel, launched just before), then each warp
-// takes single chunks from another until none is left.
+// The counters are in the workspace header (reset by zero_tiles_kernel, launched just
+// before).
 template <int W, typename Jobs>
 __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
 {
     // (what the sums go to waits in shared memory: the record loop needs the registers)
-    __shared__ volatile uint32_t s_id[RICK_GRID_WARPS], s_slot[RICK_GRID_WARPS];
-    __shared__ volatile GroupItem s_group;
+    __shared__ volatile uint32_t s_id[RICK_GRID_WARPS], s_slot[RICK_GRID_WARPS],
+        s_item[RICK_GRID_WARPS];
+    __shared__ volatile PlainWork s_work;
     const int wid = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < RICK_GRID_WARPS * SubCells<W>::CELLS; i += 32 * RICK_GRID_WARPS)
         cells[i] = make_float2(0.0f, 0.0f);
-    if (threadIdx.x == 0) s_group.slot = ~0u;
-    if (threadIdx.x < 2) s_group.total[threadIdx.x] = jobs.total(threadIdx.x);
+    if (threadIdx.x == 0) start_work(s_work, jobs.total(false), jobs.total(true));
+    s_item[wid] = ~0u;
     float2 coef2[RICK_POLY_N];
     load_coef<W>(jobs.args(0).t.kp, coef2);
     int cur = 0;
@@ -955,12 +991,14 @@ __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
     for (;;) {
         uint32_t b = 0, id, chunk, slot = ~0u;
         if (!single) {
-            b = next_group<W>(jobs, s_group);
-            single = b >= s_group.total[0];
+            b = next_group<W>(jobs, s_work);
+            single = b >= s_work.total[0];
         }
         if (single) {
-            b = next_warp(&jobs.hdr()->item_next);
-            if (b >= s_group.total[1]) break;
+            b = next_single(jobs.hdr(), s_work, s_item[wid]);
+            if (b == ~0u) break;
+            __syncwarp();
+            s_item[wid] = b;
         }
         const int j = jobs.job(b, single);
         if (single) {
@@ -973,11 +1011,11 @@ __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
             chunk = q.y + wid;
             if (q.z != ~0u) slot = q.z + q.y / RICK_SUB_GROUP % rick_sub_slots(q.w);
             if (threadIdx.x == 0) {
-                s_group.job = j;
-                s_group.id = id;
-                s_group.slot = slot;
-                s_group.first = q.z;
-                s_group.all = q.w;
+                s_work.job = j;
+                s_work.id = id;
+                s_work.slot = slot;
+                s_work.first = q.z;
+                s_work.all = q.w;
             }
         }
         const GridArgs &a = jobs.args(j);
@@ -987,15 +1025,17 @@ __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
         s_slot[wid] = slot;
         float2 *own = cells + wid * SubCells<W>::CELLS;
         grid_chunk<W>(a, id, chunk, own, coef2);
-        if (single)
+        if (single) {
             __syncwarp();
-        else
+            cells_out<W>(sub_cells(a, s_id[wid]), a.t.n, own, 1, threadIdx.x & 31, 32);
+        } else {
             __syncthreads();
-        slot = s_slot[wid];
-        cells_out<W>(slot == ~0u ? sub_cells(a, s_id[wid]) : a.slots + (size_t)slot * RICK_SLOT_CELLS,
-                     slot == ~0u ? a.t.n : RICK_SLOT_STRIDE, single ? own : cells,
-                     single ? 1 : RICK_GRID_WARPS, single ? threadIdx.x & 31 : threadIdx.x,
-                     single ? 32 : 32 * RICK_GRID_WARPS);
+            slot = s_slot[wid];
+            cells_out<W>(slot == ~0u ? sub_cells(a, s_id[wid])
+                                     : a.slots + (size_t)slot * RICK_SLOT_CELLS,
+                         slot == ~0u ? a.t.n : RICK_SLOT_STRIDE, cells, RICK_GRID_WARPS,
+                         threadIdx.x, 32 * RICK_GRID_WARPS);
+        }
         __syncwarp();
     }
 }
@@ -1089,9 +1129,9 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hdr->grid_next = 0;
         hdr->zero_next = 0;
-        hdr->item_next = 0;
         hdr->group_next = 0;
     }
+    if (blockIdx.x == 0 && threadIdx.x < RICK_ITEM_COUNTERS) hdr->item_next[threadIdx.x][0] = 0;
     const int lane = threadIdx.x & 31, T = 1 << log2T;
     if (nslots) clear_slots(hdr, slots, arrived, nslots, blockIdx.x, gridDim.x);
     if (!mcacc && accumulate) return;
@@ -1122,9 +1162,9 @@ __global__ void __launch_bounds__(256)
 {
     const GridArgs &a = ba.job[blockIdx.y];
     const TileArgs &ta = a.t;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-        ta.hdr->item_next = 0;
-        ta.hdr->group_next = 0;
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+        if (threadIdx.x == 0) ta.hdr->group_next = 0;
+        if (threadIdx.x < RICK_ITEM_COUNTERS) ta.hdr->item_next[threadIdx.x][0] = 0;
     }
     const int lane = threadIdx.x & 31;
     clear_slots(ta.hdr, a.slots, a.arrived, a.nslots, blockIdx.x, gridDim.x);

@@ -1,0 +1,74 @@
+"""Plain gridding of spread-out coverage: up to 4e5 work items of a few records, which the
+warps take one, four and eight at a time, against the compensated kernel.
+
+A cell is a sum of at most m terms in FP32, in any grouping, of the same products:
+|a - b| <= 2 (m + 4) 2^-24 S, S the sum of the terms' magnitudes.  The coverage is
+uniform, 1.5 records a subtile at most: m = 64 is far more than a cell gets.
+
+The time is asked only to be that of the compensated kernel or less: it takes six times
+the shared memory and visits the records near a tile's edge more than once.
+"""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FOV = 0.1
+
+
+def uniform(n, n_vis, dev):
+    g = torch.Generator(device=dev)
+    g.manual_seed(n_vis)
+    uvw = torch.rand((n_vis, 3), generator=g, device=dev, dtype=torch.float64) * 2.0 - 1.0
+    uvw[:, :2] *= n / 2 / FOV
+    return uvw, torch.randn(n_vis, generator=g, device=dev, dtype=torch.complex64)
+
+
+def imager(P, n, n_w, W, n_vis, precision, dev):
+    return P.Imager(n, n_w, FOV, support=W, max_vis=n_vis, device=dev, w_range=(-1.0, 1.0),
+                    precision=precision)
+
+
+@pytest.mark.parametrize("n,n_w,n_vis,W", [(512, 2, 3000, 7), (1024, 8, 40000, 5),
+                                           (2048, 8, 150000, 7), (4096, 8, 600000, 4)])
+def test_planes(n, n_w, n_vis, W):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2411_07321_gb300 as P
+    dev = torch.device("cuda", 0)
+    uvw, vis = uniform(n, n_vis, dev)
+    planes = []
+    for precision, v in (("compensated", vis), ("compensated", vis.abs() + 0j), ("fp32", vis)):
+        im = imager(P, n, n_w, W, n_vis, precision, dev)
+        im.bin(uvw, v)
+        im.planes.fill_(float("nan"))  # every cell has to be written
+        im.grid()
+        planes.append(im.planes.clone())
+        del im
+    ref, mag, got = planes
+    assert ((got - ref).abs() <= 2.0 * (64 + 4) * 2.0 ** -24 * mag.abs()).all()
+
+
+@pytest.mark.parametrize("W", [7, 9])
+def test_time(W):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2411_07321_gb300 as P
+    dev = torch.device("cuda", 0)
+    uvw, vis = uniform(2048, 1000000, dev)
+    best = {}
+    for precision in ("compensated", "fp32"):
+        im = imager(P, 2048, 8, W, len(vis), precision, dev)
+        im.bin(uvw, vis)
+        t = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            im.grid_sparse()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        best[precision] = min(t)
+        del im
+    print(W, best)
+    assert best["fp32"] <= best["compensated"]
