@@ -4,8 +4,10 @@
 // Plain gridding: one warp per work item = (subtile of one w-plane, chunk of at
 // most sub_cap records).  The warp sums the footprints of its records -- every
 // corner in the 16 x 16 cells of the subtile -- into (16 + W - 1)^2 cells of its
-// own in shared memory, with plain loads and stores, and adds the cells it
-// reached to the planes (16-byte reductions in L2) onto tiles cleared before.
+// own in shared memory, with plain loads and stores (up to W = 3 with adds), and adds
+// the cells it reached to the planes (16-byte reductions in L2) onto tiles cleared
+// before.  Eight chunks of a subtile are a CTA's, summed over its warps first; a dense
+// subtile's sums meet in slots of its own.
 //
 // Compensated and deterministic gridding: one CTA per work item = (uv-tile of
 // one w-plane, chunk of at most chunk_cap records).  The CTA owns the T x T
@@ -626,9 +628,12 @@ __device__ __forceinline__ void warp_stream(const TileArgs &ta, uint32_t r0, uin
                                             float2 *cells)
 {
     constexpr int G = StreamShape<W>::G, NGR = StreamShape<W>::NG, ST = SubCells<W>::STRIDE;
-    // Narrow kernels have eight groups a warp and more: taking turns costs more than
-    // the few compare-and-swap loops of a row.
-    constexpr bool ATOMIC = NGR > 4;
+    // Up to W = 3 a warp has ten groups and more, and taking turns costs more than the few
+    // compare-and-swap loops of a row.  Gridding of 4e6 visibilities of one channel /
+    // 1e7 of 16, adds against turns: W = 3 218 / 192 against 236 / 182 us, W = 4 290 / 209
+    // against 259 / 185, W = 5 398 / 292 against 310 / 238, W = 6 507 / 346 against 358 /
+    // 271.
+    constexpr bool ATOMIC = NGR > 8;
     using Ring = RecRing<W>;
     constexpr int RB = RICK_GRID_RB, NH = (Ring::SLOTS + 31) / 32;
     __shared__ __align__(16) float4 s_rrec[Ring::ON ? RICK_GRID_WARPS * 2 * Ring::SLOTS : 1];

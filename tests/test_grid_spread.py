@@ -49,7 +49,7 @@ def test_planes(n, n_w, n_vis, W):
     assert ((got - ref).abs() <= 2.0 * (64 + 4) * 2.0 ** -24 * mag.abs()).all()
 
 
-@pytest.mark.parametrize("W", [7, 9])
+@pytest.mark.parametrize("W", [4, 6, 7, 9])
 def test_time(W):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
