@@ -33,7 +33,8 @@ struct GridArgs {
     int log2T;
     int accumulate;  // add into the planes instead of overwriting them
     const uint8_t *touched;  // per tile: add into it (tiles an earlier chunk gridded), or NULL
-    uint32_t nzero;  // tile-clearing items (RICK_ZERO_GROUP tiles each); 0 when accumulating
+    uint32_t nzero;  // tile-clearing items (RICK_ZERO_GROUP tiles each) where every tile has
+                     // to be written, else 0 (plain sums: only whether)
     SubShape sub;            // plain sums: subtiles, their record offsets, the work items
     const uint32_t *suboff;
     const uint2 *items;
@@ -822,6 +823,25 @@ __device__ __forceinline__ void grid_chunk(const GridArgs &a, uint32_t id, uint3
     }
 }
 
+// Tile t of the planes zeroed by threads i of n_threads, 16 bytes a store.
+__device__ __forceinline__ void clear_tile(float2 *planes, uint32_t t, int nt, int log2T, int n,
+                                           int i, int n_threads)
+{
+    const uint32_t tx = t % nt, ty = t / nt % nt, k = t / nt / nt;
+    float4 *tile = (float4 *)(planes + ((size_t)k * n + (ty << log2T)) * n + (tx << log2T));
+    const int lh = log2T - 1;  // float4 = two cells
+    for (; i < 1 << (log2T + lh); i += n_threads)
+        tile[(size_t)(i >> lh) * (n / 2) + (i & ((1 << lh) - 1))] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// The tiles of [t0, t1) without records zeroed by the warp.
+__device__ __forceinline__ void clear_empty(const GridArgs &a, uint32_t t0, uint32_t t1)
+{
+    for (uint32_t t = t0; t < min(t1, a.t.ntiles); ++t)
+        if (a.t.base[t + 1] == a.t.base[t])
+            clear_tile(a.planes, t, a.t.nt, a.log2T, a.t.n, threadIdx.x & 31, 32);
+}
+
 // Two cells of a subtile's row, col even, added to its cells in the planes or a slot (row
 // stride n) -- the checkerboard (-1)^(i+j) folded in (the subtile's first row and column
 // are even); nothing where both are zero, as cells are that no footprint reached, those
@@ -888,6 +908,7 @@ __device__ __forceinline__ void cells_out(float2 *out, int n, float2 *cells, int
 struct PlainWork {
     uint32_t total[2];  // groups and single items of all jobs
     uint32_t take, idle;  // idle: CTAs without a group
+    uint32_t clear;       // tiles to look at per warp and item
     uint32_t index, id, slot, first, all;
     int job;
     bool last;
@@ -976,7 +997,13 @@ __device__ __forceinline__ uint32_t next_single(WsHeader *hdr, const volatile Pl
 
 // The counters are in the workspace header (reset by zero_tiles_kernel, launched just
 // before).
-template <int W, typename Jobs>
+//
+// CLEAR: also zero the tiles without records, a share of them with every item, so that
+// the HBM-bound clearing runs under the issue-bound gridding (as a launch of its own / so:
+// 5e7 visibilities on 32 planes of 8192^2, W = 9, 4.48 / 3.56 ms; 2e7 on 16 of 4096^2,
+// W = 7, 869 / 762 us); at the start where there are fewer items than would keep every
+// warp at it.
+template <int W, bool CLEAR, typename Jobs>
 __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
 {
     // (what the sums go to waits in shared memory: the record loop needs the registers)
@@ -988,6 +1015,19 @@ __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
         cells[i] = make_float2(0.0f, 0.0f);
     if (threadIdx.x == 0) start_work(s_work, jobs.total(false), jobs.total(true));
     s_item[wid] = ~0u;
+    if (CLEAR) {
+        __syncthreads();
+        const GridArgs &a = jobs.args(0);
+        const uint32_t warps = gridDim.x * RICK_GRID_WARPS;
+        const uint32_t items = s_work.total[0] * RICK_GRID_WARPS + s_work.total[1];
+        if (items >= 2 * warps) {
+            if (threadIdx.x == 0) s_work.clear = (a.t.ntiles + items - 1) / items;
+        } else {
+            if (threadIdx.x == 0) s_work.clear = 0;
+            for (uint32_t t = blockIdx.x * RICK_GRID_WARPS + wid; t < a.t.ntiles; t += warps)
+                clear_empty(a, t, t + 1);
+        }
+    }
     float2 coef2[RICK_POLY_N];
     load_coef<W>(jobs.args(0).t.kp, coef2);
     int cur = 0;
@@ -1041,6 +1081,12 @@ __device__ __forceinline__ void plain_work(const Jobs &jobs, float2 *cells)
                          slot == ~0u ? a.t.n : RICK_SLOT_STRIDE, cells, RICK_GRID_WARPS,
                          threadIdx.x, 32 * RICK_GRID_WARPS);
         }
+        if (CLEAR) {
+            const uint32_t per = s_work.clear;
+            const uint32_t i = single ? s_work.total[0] * RICK_GRID_WARPS + s_item[wid]
+                                      : s_work.index * RICK_GRID_WARPS + wid;
+            clear_empty(a, i * per, (i + 1) * per);
+        }
         __syncwarp();
     }
 }
@@ -1070,12 +1116,12 @@ struct OneJob {
 // W = 9: 9.21 -> 6.59; 1e7 of 4: 0.68 -> 0.35; 4e6 of one: 0.61 -> 0.33; 1e6 of 4:
 // 106 -> 52 us; 1e4: 58 -> 20 us.  Four CTAs an SM up to W = 10 (W = 9 at three:
 // 2 % slower).
-template <int W>
+template <int W, bool CLEAR>
 __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_warps_kernel(const __grid_constant__ GridArgs a)
 {
     extern __shared__ float2 s_cells[];
-    plain_work<W>(OneJob{a}, s_cells);
+    plain_work<W, CLEAR>(OneJob{a}, s_cells);
 }
 
 // Several imaging jobs gridded by one launch (rick_grid_sparse_batch): the jobs'
@@ -1089,16 +1135,6 @@ struct GridBatchArgs {
     GridArgs job[RICK_GRID_BATCH_MAX];
 };
 static_assert(sizeof(GridBatchArgs) <= 32764, "kernel parameters are limited to 32764 bytes");
-
-// Tile t of the planes zeroed by the whole block, 16 bytes a store.
-__device__ __forceinline__ void clear_tile(float2 *planes, uint32_t t, int nt, int log2T, int n)
-{
-    const uint32_t tx = t % nt, ty = t / nt % nt, k = t / nt / nt;
-    float4 *tile = (float4 *)(planes + ((size_t)k * n + (ty << log2T)) * n + (tx << log2T));
-    const int lh = log2T - 1;  // float4 = two cells
-    for (int i = threadIdx.x; i < 1 << (log2T + lh); i += blockDim.x)
-        tile[(size_t)(i >> lh) * (n / 2) + (i & ((1 << lh) - 1))] = make_float4(0.f, 0.f, 0.f, 0.f);
-}
 
 // The slots of the last binning's dense subtiles zeroed, by block b of nb.
 __device__ __forceinline__ void clear_slots(const WsHeader *hdr, float2 *slots, uint32_t *arrived,
@@ -1114,11 +1150,10 @@ __device__ __forceinline__ void clear_slots(const WsHeader *hdr, float2 *slots, 
 
 // Zero the tiles of at least `least` work items, into which the grid kernel adds,
 // before it runs, and reset its counters: least = 2 for the compensated kernel
-// (a tile's only item stores it, and the kernel itself clears the tiles without
-// records), 1 for the plain one, or 0 where every tile has to be written.
-// When gridding adds into existing planes
-// nothing is cleared, and neither are the tiles flagged in touched (a chunk of a
-// streamed set adds into the tiles earlier chunks gridded).
+// (a tile's only item stores it), 1 for the plain one.  Where every tile has to be
+// written, the grid kernels clear the tiles without records.  When gridding adds into
+// existing planes nothing is cleared, and neither are the tiles flagged in touched (a
+// chunk of a streamed set adds into the tiles earlier chunks gridded).
 // Deterministic mode (mcacc != NULL): the int64 slots of those tiles are
 // zeroed instead, accumulating or not (the slots are added into the planes
 // after gridding).
@@ -1150,7 +1185,7 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(const uint32_t *base, u
         for (; m; m &= m - 1) {
             const uint32_t t = t0 + __ffs(m) - 1;
             if (!mcacc) {
-                clear_tile(planes, t, nt, log2T, n);
+                clear_tile(planes, t, nt, log2T, n, threadIdx.x, blockDim.x);
                 continue;
             }
             ulonglong2 *slot = (ulonglong2 *)(mcacc + (size_t)mcslot[t] * 2 * T * T);
@@ -1178,7 +1213,8 @@ __global__ void __launch_bounds__(256)
         const uint32_t tl = t0 + lane;
         unsigned m = __ballot_sync(0xffffffffu, lane < RICK_ZERO_LOOK && tl < ta.ntiles &&
                                                     ta.base[tl + 1] != ta.base[tl]);
-        for (; m; m &= m - 1) clear_tile(a.planes, t0 + __ffs(m) - 1, ta.nt, a.log2T, ta.n);
+        for (; m; m &= m - 1) clear_tile(a.planes, t0 + __ffs(m) - 1, ta.nt, a.log2T, ta.n, threadIdx.x,
+                       blockDim.x);
     }
 }
 
@@ -1217,7 +1253,7 @@ __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
         }
     }
     __syncthreads();
-    plain_work<W>(BatchJobs{ba, s_cum}, s_cells);
+    plain_work<W, false>(BatchJobs{ba, s_cum}, s_cells);
 }
 
 // Deterministic mode: the tiles gridded by several work items, from their
@@ -1440,11 +1476,11 @@ static cudaError_t launch_grid(const GridArgs &a, int mode, int num_sms, cudaStr
     if (mode == GM_COMP) return launch_grid_t<W, GM_COMP>(a, num_sms, st);
     if (mode == GM_DET) return launch_grid_t<W, GM_DET>(a, num_sms, st);
     const size_t smem = warps_smem<W>();
-    cudaError_t e = cudaFuncSetAttribute(grid_warps_kernel<W>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = a.nzero ? grid_warps_kernel<W, true> : grid_warps_kernel<W, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
-    grid_warps_kernel<W><<<persistent_blocks(grid_warps_kernel<W>, smem, num_sms),
-                           32 * RICK_GRID_WARPS, smem, st>>>(a);
+    kernel<<<persistent_blocks(kernel, smem, num_sms), 32 * RICK_GRID_WARPS, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1504,7 +1540,7 @@ rick_status rick_grid_impl(rick_plan *plan, void *ws_dev, void *planes_dev, int 
     a.mcslot = det ? w.mcslot : NULL;
     a.mcacc = det ? w.mcacc : NULL;
     set_sub_args(a, p, w, L);
-    const uint32_t least = !rick_grid_plain(&p) ? 2u : mode == RICK_GRID_OVERWRITE ? 0u : 1u;
+    const uint32_t least = rick_grid_plain(&p) ? 1u : 2u;
     zero_tiles_kernel<<<(accumulate && !det && !a.nslots) ? 1 : plan->num_sms * 8, 256, 0, st>>>(
         w.gbase, a.t.ntiles, a.t.nt, a.log2T, p.n, a.planes, w.hdr, accumulate, a.mcslot,
         a.mcacc, a.touched, least, a.slots, a.arrived, a.nslots);

@@ -75,6 +75,37 @@ def test_time(W):
     assert best["fp32"] <= best["compensated"]
 
 
+def test_clearing_time():
+    """The tiles without records are cleared while the others are gridded: at least a fifth
+    of the time that clearing the planes takes is hidden."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2411_07321_gb300 as P
+    dev = torch.device("cuda", 0)
+    n, n_vis = 4096, 4000000
+    g = torch.Generator(device=dev)
+    g.manual_seed(3)
+    uvw = torch.randn((n_vis, 3), generator=g, device=dev, dtype=torch.float64)
+    uvw[:, :2] *= n / 20 / FOV
+    uvw[:, 2] = uvw[:, 2].clamp(-3.0, 3.0) / 3.0
+    vis = torch.randn(n_vis, generator=g, device=dev, dtype=torch.complex64)
+    im = imager(P, n, 16, 9, n_vis, "fp32", dev)
+    im.bin(uvw, vis)
+    best = {}
+    for name, f in (("sparse", im.grid_sparse), ("dense", im.grid), ("zero", im.planes.zero_)):
+        t = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            f()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        best[name] = min(t)
+    print(best)
+    assert best["dense"] <= best["sparse"] + 0.8 * best["zero"]
+
+
 def test_binning_time():
     """Building the lists of a million items costs the binning less than two fifths of what
     the same number of visibilities on a sixteenth of each side takes."""
