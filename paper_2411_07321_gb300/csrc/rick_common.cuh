@@ -823,12 +823,12 @@ rick_status rick_grid_impl(rick_plan *plan, void *ws_dev, void *planes_dev, int 
 bool rick_fft_tables(rick_plan *pl);
 // Bytes of the fused transform's work buffer (0 where it does not cover n).
 size_t rick_fft_work_bytes(const rick_params *p);
-// Tiles the fused transform reads (mode 0: all; 1: this binning's; 2: add this
-// binning's to those marked), kept in the work buffer.
+// Tiles the fused transform reads, kept in the work buffer: this binning's, or with add
+// these besides those marked.
 rick_status rick_fft_tiles_impl(rick_plan *plan, const void *ws_dev, void *work_dev,
-                                size_t work_bytes, int mode, cudaStream_t st);
-// The fused inverse FFT + w-correction of the marked tiles (tiles -1), or after
-// marking them as rick_fft_tiles_impl's mode 0 or 1 does.
+                                size_t work_bytes, int add, cudaStream_t st);
+// The fused inverse FFT + w-correction of the marked tiles (tiles -1), after marking
+// this binning's (1), or of every tile (0).
 rick_status rick_fft_wcorrect_impl(rick_plan *plan, const void *planes_dev, const void *ws_dev,
                                    void *work_dev, size_t work_bytes, float *image_dev,
                                    uint32_t flags, cudaStream_t st, int tiles = -1);

@@ -290,8 +290,8 @@ static __device__ __forceinline__ void load_sel(float2 (&x)[16], const float2 *s
 // half the planes are transformed; the middle one of an odd number is its own
 // opposite (w = 0) and goes alone.
 //
-// FOLD: the kernels for plans whose range is symmetric (the binning's decides); the
-// others are without it (its registers cost the row pass of n = 8192 7 %).  16 planes
+// FOLD: the kernels for plans whose range is symmetric (the binning's decides) on grids
+// that fill the GPU (launch_fft_wc); the others are without it (its registers cost the row pass of n = 8192 7 %).  16 planes
 // of 4096^2, 32e6 visibilities in the streamed call: rows 506 -> 370 us, columns 871
 // -> 555; both sides' tile-rows are read for the half of the planes.
 template <bool FOLD>
@@ -383,21 +383,22 @@ struct XLen {
     static constexpr int L = N + N / 16;
 };
 
-// Tiles to read: a tile holds records iff it has gridding work items.
-// mode 0: every tile; 1: the tiles of this binning; 2: add this binning's
-// tiles to those already marked (planes gridded over several binnings).
+// Tiles to read: a tile holds records iff it has gridding work items.  The tiles of
+// this binning, or with add these besides those already marked (planes gridded over
+// several binnings).
 __global__ void __launch_bounds__(256) fft_tiles_kernel(uint8_t *tflag, const uint32_t *gbase,
-                                                        uint32_t ntiles, int mode)
+                                                        uint32_t ntiles, int add)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ntiles) return;
-    const uint8_t has = mode == 0 || gbase[t + 1] != gbase[t];
-    tflag[t] = mode == 2 ? (uint8_t)(tflag[t] | has) : has;
+    const uint8_t has = gbase[t + 1] != gbase[t];
+    tflag[t] = add ? (uint8_t)(tflag[t] | has) : has;
 }
 
 // Tile-rows and planes with a tile to read: one block of 32 warps per plane, a warp
-// per tile-row at a time (with eight warps, 30 us of load latency at 128 a side).  gbase (optional): the tiles are this binning's (or with all, every
-// one), and their flags are written first; else the flags are there.
+// per tile-row at a time (with eight warps, 30 us of load latency at 128 a side).
+// gbase (optional): the tiles are this binning's (or with all, every one), and their
+// flags are written first; else the flags are there.
 __global__ void __launch_bounds__(1024) fft_rowflags_kernel(FftArgs a, const uint32_t *gbase, int all)
 {
     const int k = blockIdx.x, nt = a.nt, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1004,6 +1005,16 @@ static cudaError_t launch_fft_wc(const FftArgs &a, bool fold, int num_sms, cudaS
 {
     using S = ColShape<LOGN>;
     using RS = RowShape<(1 << LOGN)>;
+    const int m = a.wc.m, ctas = (m + S::COLS - 1) / S::COLS;
+    // planes split over clusters of up to 8 CTAs, and of no more than there are planes,
+    // while all of them are resident at once (two a SM up to n = 4096)
+    int split = 1;
+    const int room = num_sms * (S::NT <= 256 ? 2 : 1);
+    while (split < 8 && 2 * split <= a.n_w && ctas * 2 * split <= room) split *= 2;
+    // Grids that split do not fold: half the planes one after the other take longer than
+    // all of them side by side (whole transform, folded / split: 2 planes of 256^2 31 / 28
+    // us, 9 37 / 27; 3 of 512^2 35 / 33, 8 42 / 37).
+    if (split > 1) fold = false;
     const size_t rows_smem = sizeof(float2) * RS::ROWS * XLen<(1 << LOGN)>::L;
     const auto rows = fold ? fft_rows_kernel<LOGN, true> : fft_rows_kernel<LOGN, false>;
     cudaError_t e = fft_smem_attrs(rows, rows_smem);
@@ -1012,12 +1023,6 @@ static cudaError_t launch_fft_wc(const FftArgs &a, bool fold, int num_sms, cudaS
     rows<<<(unsigned)min(items, num_sms * RS::PER_SM), RS::NT, rows_smem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int m = a.wc.m, ctas = (m + S::COLS - 1) / S::COLS;
-    // planes split over clusters of up to 8 CTAs while all of them are resident at once
-    // (two a SM up to n = 4096) and each keeps a plane
-    int split = 1;
-    const int room = num_sms * (S::NT <= 256 ? 2 : 1);
-    while (!fold && split < 8 && 2 * split <= a.n_w && ctas * 2 * split <= room) split *= 2;
     const auto cols = fold ? fft_cols_kernel<LOGN, false, true>
                     : split == 1 ? fft_cols_kernel<LOGN, false, false>
                                  : fft_cols_kernel<LOGN, true, false>;
@@ -1075,7 +1080,7 @@ static FftArgs fft_args(rick_plan *plan, const void *ws_dev, void *work_dev, uin
 }
 
 rick_status rick_fft_tiles_impl(rick_plan *plan, const void *ws_dev, void *work_dev,
-                                size_t work_bytes, int mode, cudaStream_t st)
+                                size_t work_bytes, int add, cudaStream_t st)
 {
     if (!fft_args_ok(plan, ws_dev, work_dev, work_bytes)) return RICK_EINVAL;
     const rick_params &p = plan->p;
@@ -1083,7 +1088,7 @@ rick_status rick_fft_tiles_impl(rick_plan *plan, const void *ws_dev, void *work_
     WsPtrs wp = rick_ws_ptrs((void *)ws_dev, rick_ws_layout(&p, plan->max_vis));
     const uint32_t nt = p.n / p.tile, ntiles = (uint32_t)p.n_w * nt * nt;
     fft_tiles_kernel<<<(ntiles + 255) / 256, 256, 0, st>>>((uint8_t *)work_dev + L.tflag,
-                                                           wp.gbase, ntiles, mode);
+                                                           wp.gbase, ntiles, add);
     RICK_LAUNCH_CHECK(plan);
     return RICK_OK;
 }

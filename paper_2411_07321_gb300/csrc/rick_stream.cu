@@ -273,8 +273,7 @@ static rick_status stream_impl(rick_plan *plan, int64_t n_units, int32_t n_chan,
                                     c > 0 ? RICK_GRID_ACCUMULATE : RICK_GRID_OVERWRITE, st));
         // the tiles this chunk's records reach, for the fused transform
         if (S.fwork_bytes)
-            RICK_TRY(rick_fft_tiles_impl(plan, ws_dev, sb + S.fwork, S.fwork_bytes, c > 0 ? 2 : 1,
-                                         st));
+            RICK_TRY(rick_fft_tiles_impl(plan, ws_dev, sb + S.fwork, S.fwork_bytes, c > 0, st));
     }
     // every binning of this call has read its resident uvw area and factors
     RICK_CUDA_TRY(plan, cudaEventRecord(plan->ev_area_free[area], st));
