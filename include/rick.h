@@ -316,8 +316,9 @@ rick_status rick_bin_values(rick_plan *plan, const void *vis_dev, const float *w
                             void *ws_dev, rick_bin_stats *stats_dev, void *stream);
 
 /* chi^2 = sum_m w_m |vis_m - model_m|^2 over n_vis visibilities, and the residuals
- * vis - model in place of the model.  The sum is taken in FP64, in an order that
- * depends on n_vis alone.
+ * vis - model in place of the model.  Terms are FP32; a thread's are added in FP32
+ * pairs (double-single; where that overflows, in plain FP32, to infinity), the
+ * threads' sums in FP64, in an order that depends on n_vis alone.
  *   vis_dev, weight_dev: complex64 and float32 [n_vis] (weight not NULL)
  *   model_dev:           complex64 [n_vis], overwritten with the residuals
  *   partials_dev:        scratch of RICK_CHI2_PARTIALS float64

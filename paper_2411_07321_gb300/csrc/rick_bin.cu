@@ -1406,8 +1406,10 @@ __global__ void __launch_bounds__(256) chi2_residuals_kernel(int64_t n, const fl
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     // four visibilities in flight; their FP32 terms are added in FP32 pairs of
-    // double-single first (FP64 issues at a sixty-fourth of the rate)
+    // double-single first (FP64 issues at a sixty-fourth of the rate), and in plain FP32
+    // for sums that are not finite, of which a pair makes NaN (inf - inf)
     ff acc = {0.0f, 0.0f};
+    float plain = 0.0f;
     for (; i < n; i += 4 * step) {
         float2 o[4], m[4];
         float w[4];
@@ -1430,9 +1432,10 @@ __global__ void __launch_bounds__(256) chi2_residuals_kernel(int64_t n, const fl
             model[j] = r;
             const float e = w[u] * __fadd_rn(__fmul_rn(r.x, r.x), __fmul_rn(r.y, r.y));
             acc = ff_add(acc, ff{e, 0.0f});
+            plain += e;
         }
     }
-    t = (double)acc.hi + (double)acc.lo;
+    t = isfinite(acc.hi) ? (double)acc.hi + (double)acc.lo : (double)plain;
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = t;
     __syncthreads();
