@@ -76,9 +76,14 @@ class Chi2Fn(torch.autograd.Function):
         return ctx.imager.image_from_binned(ctx.flags), None, None, None, None
 
 
+def _known(t) -> bool:
+    """A tensor or a module's parameter, and no other kind of tensor."""
+    return type(t) in (torch.Tensor, torch.nn.Parameter)
+
+
 def _plain(t, dtype, shape, device) -> bool:
     """A tensor the library can take as it is, and that asks for no gradient."""
-    return (type(t) is torch.Tensor and t.dtype == dtype and tuple(t.shape) == shape
+    return (_known(t) and t.dtype == dtype and tuple(t.shape) == shape
             and t.device == device and t.is_contiguous() and not t.requires_grad
             and not t.is_conj() and not t.is_neg())
 
@@ -98,7 +103,7 @@ def chi2(image, imager, vis_obs, weight):
     torch operations on the model visibilities, in vis_obs and weight)."""
     n = (imager.n_vis,)
     if (n[0] > 0 and forward_ad._current_level < 0  # no forward-mode tangents
-            and type(image) is torch.Tensor and image.dtype == torch.float32
+            and _known(image) and image.dtype == torch.float32
             and not image.is_neg()
             and _plain(vis_obs, torch.complex64, n, imager.device)
             and _plain(weight, torch.float32, n, imager.device)):

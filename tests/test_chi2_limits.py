@@ -46,6 +46,22 @@ def test_not_finite(n_vis, at, value):
     assert math.isnan(float(want)) or float(loss.detach()) == float(want)
 
 
+def test_parameter():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    im, A, vis, w = setup(3000)
+    g = torch.Generator(device=vis.device)
+    g.manual_seed(1)
+    x = torch.randn((256, 256), generator=g, device=vis.device)
+    grads = []
+    for image in (torch.nn.Parameter(x.clone()), x.clone().requires_grad_()):
+        loss = A.chi2(image, im, vis, w)
+        assert type(loss.grad_fn).__name__ == "Chi2FnBackward"
+        loss.backward()
+        grads.append(image.grad)
+    assert float((grads[0] - grads[1]).abs().max()) <= 1e-5 * float(grads[1].abs().max())
+
+
 @pytest.mark.parametrize("n_vis", [(1 << 20) + 1, (1 << 21) + 12345])
 def test_more_than_a_round(n_vis):
     """Against an FP64 sum of the terms of the same FP32 residuals: three roundings of a
