@@ -1111,14 +1111,13 @@ struct OneJob {
 // and stores of 8 bytes a lane, and only the groups meet at barriers; summing a
 // 64 x 64 tile per CTA took 2 W compare-and-swap loops a lane there (shared memory
 // has no FP32 add) and visited the records near a tile's edge once per tile they
-// reach.  16 x 16 corners a subtile leave 32 warps an SM, 24 of the wider kernels.  On
-// a GB300, against the CTA tiles: 5e7 visibilities of 16 channels, W = 7: 1.92 -> 1.26
-// ms; 2e8 of 64, W = 9: 9.21 -> 6.45; 1e7 of 4: 0.68 -> 0.36; 4e6 of one: 0.61 -> 0.34;
-// 1e6 of 4: 106 -> 57 us; 1e4: 58 -> 17 us.  Four CTAs an SM up to W = 8; wider kernels spill at
-// 64 registers (four / three: 4e6 visibilities of one channel, W = 9 591 / 548 us, W = 10
-// 634 / 588; 1e7 of 16 431 / 419, 457 / 436).
+// reach.  16 x 16 corners a subtile leave 32 warps an SM.  On a GB300, against the
+// CTA tiles: 5e7 visibilities of 16 channels, W = 7: 1.92 -> 1.24 ms; 2e8 of 64,
+// W = 9: 9.21 -> 6.59; 1e7 of 4: 0.68 -> 0.35; 4e6 of one: 0.61 -> 0.33; 1e6 of 4:
+// 106 -> 52 us; 1e4: 58 -> 20 us.  Four CTAs an SM up to W = 10 (W = 9 at three:
+// 2 % slower).
 template <int W, bool CLEAR>
-__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 8 ? 4 : 3)
+__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_warps_kernel(const __grid_constant__ GridArgs a)
 {
     extern __shared__ float2 s_cells[];
@@ -1239,7 +1238,7 @@ struct BatchJobs {
 
 // As grid_warps_kernel over the batch's work.
 template <int W>
-__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 8 ? 4 : 3)
+__global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_batch_kernel(const __grid_constant__ GridBatchArgs ba)
 {
     extern __shared__ float2 s_cells[];
