@@ -970,10 +970,11 @@ struct SubEntries {
 };
 __device__ __forceinline__ SubEntries reserve_items(uint32_t cnt, uint32_t *len)
 {
-    SubEntries e;
+    SubEntries e = {};
+    e.slot = ~0u;
+    if (!__any_sync(FULL, cnt != 0)) return e;
     e.ng = cnt / RICK_SUB_GROUP;
     const uint32_t ns = rick_sub_slots(e.ng);
-    e.slot = ~0u;
     if (__any_sync(FULL, ns != 0)) {
         const uint32_t at = reserve(ns, len + 2).lane;
         if (ns) e.slot = at;

@@ -1112,10 +1112,12 @@ struct OneJob {
 // 64 x 64 tile per CTA took 2 W compare-and-swap loops a lane there (shared memory
 // has no FP32 add) and visited the records near a tile's edge once per tile they
 // reach.  16 x 16 corners a subtile leave 32 warps an SM.  On a GB300, against the
-// CTA tiles: 5e7 visibilities of 16 channels, W = 7: 1.92 -> 1.24 ms; 2e8 of 64,
-// W = 9: 9.21 -> 6.59; 1e7 of 4: 0.68 -> 0.35; 4e6 of one: 0.61 -> 0.33; 1e6 of 4:
-// 106 -> 52 us; 1e4: 58 -> 20 us.  Four CTAs an SM up to W = 10 (W = 9 at three:
-// 2 % slower).
+// CTA tiles: 5e7 visibilities of 16 channels, W = 7: 1.92 -> 1.27 ms; 2e8 of 64,
+// W = 9: 9.21 -> 6.57; 1e7 of 4: 0.68 -> 0.36; 4e6 of one: 0.61 -> 0.34; 1e6 of 4:
+// 106 -> 57 us; 1e4: 58 -> 17 us.  Four CTAs an SM up to W = 10, where 64 registers
+// spill: long runs want the warps, short ones do not (four / three, W = 9: 2e8 of 64
+// channels 6.57 / 6.80 ms, 6e6 of 64 247 / 240 us, 4e6 of one 591 / 548, 1e7 of 16 431 /
+// 419; W = 10: 634 / 588, 457 / 436).  From W = 11 three (W = 11 at four: 386 / 407).
 template <int W, bool CLEAR>
 __global__ void __launch_bounds__(32 * RICK_GRID_WARPS, W <= 10 ? 4 : 3)
     grid_warps_kernel(const __grid_constant__ GridArgs a)
