@@ -340,12 +340,13 @@ rick_status rick_bin_residuals(rick_plan *plan, const void *resid_dev, const flo
  * checkerboard (-1)^(i+j) of the centred FFT folded in.  Every element of
  * planes_dev (complex64 [n_w][n][n]) is overwritten.  Records are summed
  * in shared memory, by subtiles of 16 x 16 corners, and the sums added to the
- * cleared planes with float atomics (compensated and deterministic plans: by
- * uv-tiles, each written once unless it has more records than one chunk).  The kernel
+ * cleared planes with float atomics; the partial sums of a dense subtile are
+ * first added up in FP64 (compensated and deterministic plans: by uv-tiles,
+ * each written once unless it has more records than one chunk).  The kernel
  * weights G are degree-8 polynomial fits per unit segment (FP64 fit at plan
- * creation, FP32 evaluation).  rick_grid and rick_degrid use a word of the
- * workspace header as a work counter: calls that share a workspace must not
- * overlap on the device. */
+ * creation, FP32 evaluation).  rick_grid and rick_degrid keep their work
+ * counters and the dense subtiles' sums in the workspace: calls that share one
+ * must not overlap on the device. */
 rick_status rick_grid(rick_plan *plan, void *ws_dev, void *planes_dev, void *stream);
 
 /* rick_grid that adds into planes_dev instead of overwriting it: planes_dev
@@ -354,8 +355,8 @@ rick_status rick_grid(rick_plan *plan, void *ws_dev, void *planes_dev, void *str
  * chunks of a visibility set one after another -- rick_bin + rick_grid for
  * the first, rick_bin + rick_grid_accumulate for the rest, all binned with the
  * same w range -- gives the planes of the whole set (up to FP32 summation
- * order).  Tiles written by one work item are read, added to and written;
- * tiles of several work items add with float atomics. */
+ * order).  Every sum is added with float atomics (compensated and
+ * deterministic plans: a tile of one work item is read, added to and written). */
 rick_status rick_grid_accumulate(rick_plan *plan, void *ws_dev, void *planes_dev, void *stream);
 
 /* Per-plane 2D FFT (§2 step 3, §3.1): cuFFT complex64, unnormalised, in place,
@@ -385,7 +386,7 @@ rick_status rick_wcorrect_stack(rick_plan *plan, const void *planes_dev, const v
 rick_status rick_grid_sparse(rick_plan *plan, void *ws_dev, void *planes_dev, void *stream);
 
 /* rick_grid_sparse of n_jobs imaging jobs in one launch (§2 step 2, Eq. 3, for
- * each job): the work items (uv-tile, chunk of records) of every job's last
+ * each job): the work items (chunks of a subtile's records) of every job's last
  * rick_bin form one list, which one persistent grid kernel works through.  For
  * serving many small jobs, whose own launches would each leave most of the GPU
  * idle.  plans[j], ws_dev[j], planes_dev[j]: job j's plan, the workspace of its
@@ -397,7 +398,7 @@ rick_status rick_grid_sparse(rick_plan *plan, void *ws_dev, void *planes_dev, vo
  * in another order).  Enqueued on stream; the caller orders it after every
  * job's binning (and before what reads the planes).  A CUDA launch error marks
  * every plan of the batch with RICK_ECUDA.  Uses the first job's workspace
- * header as the batch's work counter. */
+ * header for the batch's work counters. */
 #define RICK_GRID_BATCH_MAX 16
 rick_status rick_grid_sparse_batch(rick_plan *const *plans, void *const *ws_dev,
                                    void *const *planes_dev, int32_t n_jobs, void *stream);
@@ -415,7 +416,9 @@ rick_status rick_fused_work_bytes(const rick_params *params, size_t *work_bytes)
  * uint8 plane flags [n_w], 128-bit tile-row bit masks [n_w] and tile bit
  * masks [n_w][nt] (two uint64 each, for nt <= 128), then the row transforms, complex64
  * [n_w][image_n][n] (8 n_w image_n n bytes; image_n = n without a crop; at
- * n = 8192 the columns are stored in interleaved pairs, [n_w][image_n/2][n][2]).
+ * n = 4096 and 8192 the columns are stored in interleaved pairs,
+ * [n_w][image_n/2][n][2]).  Where opposite planes are folded (see
+ * rick_fft_wcorrect) the planes of the upper half hold nothing.
  * RICK_EINVAL if n is outside 256 ... 8192, the sizes the fused transform
  * covers (use rick_fft_wplanes + rick_wcorrect_stack there). */
 rick_status rick_fft_wcorrect_bytes(const rick_plan *plan, size_t *work_bytes);
@@ -427,15 +430,20 @@ rick_status rick_fft_wcorrect_bytes(const rick_plan *plan, size_t *work_bytes);
  * Two passes of 1D transforms: along u for the rows of tile-rows that hold
  * records, stored transposed in work_dev; then along v for each image column,
  * summing the planes into the image (the w-phase of each block of 8 planes
- * by Horner's rule from the block's exact first-plane phase).
+ * by Horner's rule from the block's exact first-plane phase).  On grids with too
+ * few columns to fill the GPU the planes are split over a cluster of CTAs, whose
+ * sums are added in rank order.  With a w range symmetric about zero, plane
+ * n_w - 1 - k has the centre -w_k, so its cells are folded into plane k's (their
+ * conjugate at the opposite cell) and the two are transformed as one.
  *   sparse = 1: only the tiles with gridding work items in ws_dev are read;
  *               all other tiles are taken as zero (planes_dev from rick_grid
  *               or rick_grid_sparse with this ws_dev).
  *   sparse = 0: every tile is read (planes accumulated over several binnings).
  * work_dev: device, 256-byte aligned, at least rick_fft_wcorrect_bytes; its
  * contents are scratch, and calls that share it must not overlap on the device.
- * ws_dev supplies the w range, the weight sum and (for sparse) the tiles.  RICK_EINVAL for an n outside 256 ... 8192, a short or
- * misaligned buffer or unknown flags. */
+ * ws_dev supplies the w range, the weight sum and (for sparse) the tiles.
+ * RICK_EINVAL for an n outside 256 ... 8192, a short or misaligned buffer or
+ * unknown flags. */
 rick_status rick_fft_wcorrect(rick_plan *plan, const void *planes_dev, const void *ws_dev,
                               int32_t sparse, void *work_dev, size_t work_bytes,
                               float *image_dev, uint32_t flags, void *stream);

@@ -150,9 +150,10 @@ struct WsLayout {
 // support is at most 16: one per row of subtiles), of class 2 (the last subtile)
 // and of class 3 (one per column).  The histogram counts sub-bins; the value a
 // counter held before an input's atomic is the input's rank in its sub-bin.
-// Several counters per sub-bin, to spread the atomics of the densest ones, gain
-// nothing (LOFAR-like 5e7 visibilities: key pass 593 us with one counter per
-// bin, 596 with eight, 597 with 32).
+// Where many warps reach the same few counters, their atomics hold the pass up:
+// 5e7 visibilities of 16 channels take 604 us, with a sixth of them in one tile
+// 1070.  (Adding up in the block's shared memory first takes 690 us there and half
+// the time on single-channel sets, but 2 to 10 % longer on all others.)
 #define RICK_SUB_LOG 4
 
 struct SubShape {

@@ -291,9 +291,10 @@ static __device__ __forceinline__ void load_sel(float2 (&x)[16], const float2 *s
 // opposite (w = 0) and goes alone.
 //
 // FOLD: the kernels for plans whose range is symmetric (the binning's decides) on grids
-// that fill the GPU (launch_fft_wc); the others are without it (its registers cost the row pass of n = 8192 7 %).  16 planes
-// of 4096^2, 32e6 visibilities in the streamed call: rows 506 -> 370 us, columns 871
-// -> 555; both sides' tile-rows are read for the half of the planes.
+// that fill the GPU (launch_fft_wc); the others are without it (its registers cost the
+// row pass of n = 8192 7 %).  16 planes of 4096^2, 32e6 visibilities in the streamed
+// call: rows 506 -> 370 us, columns 871 -> 555; both sides' tile-rows are read for the
+// half of the planes.
 template <bool FOLD>
 struct Fold {
     int planes;  // planes to transform

@@ -225,7 +225,8 @@ class Imager:
     def fused_tiles(self, planes: bool = False):
         """(plane, uv-tile) and (plane, tile-row) pairs the last fft_wcorrect read
         (from the flags at the head of its work buffer); with ``planes`` also the
-        number of planes it transformed."""
+        number of planes it read.  Where the w range is symmetric about zero it may
+        have transformed opposite planes as one, half as many transforms."""
         if self._fwork is None:
             return (0, 0, 0) if planes else (0, 0)
         nt = self.n // self.params.tile
