@@ -137,9 +137,11 @@ def probe_rates(P) -> dict:
 def stage_rooflines(wl, m: dict, rates: dict, sms: int, sm_mhz: float, hbm_peak: float) -> dict:
     """Each stage against the unit that bounds it:
     - bin: HBM (algorithmic bytes / measured copy bandwidth);
-    - grid: shared memory -- Eq. 3 accumulates 2 W^2 FP32 values per visibility;
-      the peak is the measured plain read-modify-write rate of shared memory
-      (the faster of the two ways to add into it); HBM bytes alongside;
+    - grid: FP32 multiply-adds -- Eq. 3 takes 2 W^2 of them per visibility (re and
+      im of W^2 cells), 4 W^2 flops, against the measured FP32 FMA rate; HBM bytes
+      alongside.  The rate of 2 W^2 shared-memory read-modify-writes per visibility
+      is reported too, as a normalised rate: sums that stay in registers while the
+      footprint does not move need none, so it bounds nothing;
     - fft_wcorrect: FP32 arithmetic -- 5 N log2 N flops per N-point complex
       transform (the usual count), one per row of the tile-rows with records
       plus one per image column and plane with records, against the measured
@@ -151,26 +153,24 @@ def stage_rooflines(wl, m: dict, rates: dict, sms: int, sm_mhz: float, hbm_peak:
     hb = {k: alg[k] / (ms[k] * 1e-3) / 1e9 for k in ms}
     out["bin"] = {"bound": "hbm", "achieved": hb["bin"], "peak": hbm_peak, "unit": "GB/s",
                   "frac": hb["bin"] / hbm_peak, "work": alg["bin"]}
-    smem_ops = 2 * wl.support ** 2 * m["n_binned"]
-    smem_peak = rates["smem_rmw_f32"] * sms * clk
-    g = smem_ops / (ms["grid"] * 1e-3)
-    out["grid"] = {"bound": "smem", "achieved": g / 1e9, "peak": smem_peak / 1e9,
-                   "unit": "G FP32 shared read-modify-writes/s", "frac": g / smem_peak,
-                   "work": smem_ops, "hbm_frac": hb["grid"] / hbm_peak,
-                   "peak_note": f"{rates['smem_rmw_f32']:.2f} RMW/clk/SM measured x {sms} SMs x "
-                                f"{sm_mhz:.0f} MHz"}
+    fma = max(rates["ffma"], rates["ffma2"])  # the faster of single and paired FMAs
+    fpeak = 2.0 * fma * sms * clk
+    fnote = (f"{fma:.1f} FP32 FMA/clk/SM measured x 2 flops x {sms} SMs x {sm_mhz:.0f} MHz")
+    cells = 2 * wl.support ** 2 * m["n_binned"]  # values added up
+    g = cells / (ms["grid"] * 1e-3)
+    out["grid"] = {"bound": "alu", "achieved": 2 * g / 1e12, "peak": fpeak / 1e12,
+                   "unit": "TFLOP/s (FP32)", "frac": 2 * g / fpeak, "work": 2 * cells,
+                   "hbm_frac": hb["grid"] / hbm_peak, "peak_note": fnote,
+                   "per_smem_rmw_rate": g / (rates["smem_rmw_f32"] * sms * clk)}
     n = wl.n
     m_img = n
     transforms = m["tile_rows"] * wl.tile + m_img * m["planes_read"]
     flops = 5.0 * n * math.log2(n) * transforms
-    fma = max(rates["ffma"], rates["ffma2"])  # the faster of single and paired FMAs
-    fpeak = 2.0 * fma * sms * clk
     f = flops / (ms["fft_wcorrect"] * 1e-3)
     out["fft_wcorrect"] = {"bound": "alu", "achieved": f / 1e12, "peak": fpeak / 1e12,
                            "unit": "TFLOP/s (FP32)", "frac": f / fpeak, "work": flops,
                            "hbm_frac": hb["fft_wcorrect"] / hbm_peak,
-                           "peak_note": f"{fma:.1f} FP32 FMA/clk/SM measured x 2 flops x "
-                                        f"{sms} SMs x {sm_mhz:.0f} MHz"}
+                           "peak_note": fnote}
     return out
 
 
