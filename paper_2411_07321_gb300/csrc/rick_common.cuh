@@ -240,10 +240,14 @@ RICK_HD uint32_t rick_sub_slots(uint32_t groups)
     return groups < RICK_SLOT_GROUPS ? 0 : groups < 8 * 16 ? (groups + 7) / 8 : 16;
 }
 RICK_HD uint32_t rick_sub_chunks(uint32_t n, uint32_t cap) { return (n + cap - 1) / cap; }
+static inline int64_t rick_sub_least(int64_t n_vis, int num_sms)
+{
+    const int64_t least = n_vis / ((int64_t)num_sms * 32);
+    return least < RICK_SUB_CAP_MIN ? RICK_SUB_CAP_MIN : least > 128 ? 128 : least;
+}
 static inline uint32_t rick_sub_cap(int64_t n_vis, int num_sms)
 {
-    int64_t least = n_vis / ((int64_t)num_sms * 32);
-    least = least < RICK_SUB_CAP_MIN ? RICK_SUB_CAP_MIN : least > 128 ? 128 : least;
+    const int64_t least = rick_sub_least(n_vis, num_sms);
     int64_t c = n_vis / ((int64_t)num_sms * 128);
     c = c < least ? least : c > RICK_SUB_CAP_MAX ? RICK_SUB_CAP_MAX : c;
     return (uint32_t)((c + 31) & ~(int64_t)31);
@@ -313,7 +317,10 @@ static inline WsLayout rick_ws_layout(const rick_params *p, int64_t n_vis_in)
         if (L.nitems > n_vis) L.nitems = n_vis;
         L.nitems += n_vis / RICK_SUB_CAP_MIN + 1;
         L.ngroups = n_vis / (RICK_SUB_GROUP - 1) / RICK_SUB_CAP_MIN + 1;
-        L.nslots = 2 * L.ngroups / RICK_SLOT_GROUPS;
+        // slots: 8 KB each, so by the chunk length of a full GPU's work (152 SMs; with
+        // other counts the last subtiles may go without)
+        L.nslots = 2 * (n_vis / (RICK_SUB_GROUP - 1) / rick_sub_least(n_vis, 152)) /
+                   RICK_SLOT_GROUPS;
         if (L.nslots > RICK_SLOTS_MAX) L.nslots = RICK_SLOTS_MAX;
     }
     L.nscan = rick_scan_tmp(L.nsubs + 1);
